@@ -563,7 +563,8 @@ dp_status dp_field_load(dp_ctx *ctx, const double *links, const int dims[4], int
     f->g = g;
     f->bc_t = bc_t;
     double2 *lex = (double2 *)c.alloc(n * sizeof(double));
-    bool ok = lex != nullptr;
+    int *flag = (int *)c.alloc(sizeof(int));
+    bool ok = lex != nullptr && flag != nullptr;
     for (int p = 0; p < 2 && ok; p++) {
         f->l64[p] = (double2 *)c.alloc(g.Vh * 4 * 9 * sizeof(double2));
         f->l32f[p] = (float2 *)c.alloc(g.Vh * 4 * 9 * sizeof(float2));
@@ -572,6 +573,7 @@ dp_status dp_field_load(dp_ctx *ctx, const double *links, const int dims[4], int
     }
     if (!ok) {
         c.release(lex);
+        c.release(flag);
         for (int p = 0; p < 2; p++) {
             c.release(f->l64[p]);
             c.release(f->l32f[p]);
@@ -581,10 +583,15 @@ dp_status dp_field_load(dp_ctx *ctx, const double *links, const int dims[4], int
         return DP_ERR_OOM;
     }
     CUDA_OK(cudaMemcpyAsync(lex, links, n * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-    CUDA_OK(launch_pack_links(lex, g, f->l64, f->l32f, f->l32c, c.stream));
+    CUDA_OK(cudaMemsetAsync(flag, 0, sizeof(int), c.stream));
+    CUDA_OK(launch_pack_links(lex, g, f->l64, f->l32f, f->l32c, flag, c.stream));
     c.launches++;
+    int odd = 0;
+    CUDA_OK(cudaMemcpyAsync(&odd, flag, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     CUDA_OK(cudaStreamSynchronize(c.stream));
+    f->unitary = odd == 0;
     c.release(lex);
+    c.release(flag);
     std::lock_guard<std::mutex> lk(c.mu);
     const uint64_t id = c.next_field++;
     c.fields[id] = f;
@@ -724,6 +731,9 @@ dp_status dp_apply(dp_ctx *ctx, dp_field field, int kind, double M, const dp_pro
     void *ie = c.alloc(vb), *io = c.alloc(vb), *oe = c.alloc(vb), *oo = c.alloc(vb);
     void *te = c.alloc(vb), *to = c.alloc(vb);
     void *hopd = c.alloc(hop.size() * sizeof(double));
+    // FP64 hops: exponents for the integer kernel (without them the FP64 kernel serves)
+    const bool hops = kind == DP_APPLY_HOP || kind == DP_APPLY_FULL;
+    int *ex = hops && pr == 0 && f.unitary ? (int *)c.alloc((size_t)g.V * nk * sizeof(int)) : nullptr;
     dp_status ret = DP_OK;
     if (!lex || !ie || !io || !oe || !oo || !te || !to || !hopd) {
         set_error("out of device memory (dp_apply)");
@@ -741,7 +751,7 @@ dp_status dp_apply(dp_ctx *ctx, dp_field field, int kind, double M, const dp_pro
                 CUDA_OK(cudaMemcpyAsync(hopd, hopf.data(), hopf.size() * sizeof(float),
                                         cudaMemcpyHostToDevice, c.stream));
             void *inp[2] = {ie, io}, *outp[2] = {oe, oo}, *tmp[2] = {te, to};
-            for (int p = 0; p < 2; p++) {
+            for (int p = 0; p < 2 && kind != DP_APPLY_HOP; p++) {
                 const void *mat;
                 if (kind == DP_APPLY_CLOVER_INV)
                     mat = pr == 0 ? (const void *)ci->inv64[p] : (const void *)ci->inv32[p];
@@ -754,32 +764,31 @@ dp_status dp_apply(dp_ctx *ctx, dp_field field, int kind, double M, const dp_pro
                 cp.nrhs = nk;
                 cp.in = inp[p];
                 cp.out = (kind == DP_APPLY_FULL) ? tmp[p] : outp[p];
-                if (kind == DP_APPLY_CLOVER || kind == DP_APPLY_CLOVER_INV) {
-                    CUDA_OK(launch_clover_apply(cp, pr, c.stream));
-                    continue;
-                }
+                CUDA_OK(launch_clover_apply(cp, pr, c.stream));
+            }
+            int *exp[2] = {ex, ex ? ex + (size_t)g.Vh * nk : nullptr};
+            for (int p = 0; p < 2 && ex; p++)  // (the inputs are not read again)
+                CUDA_OK(launch_to_fx((const double2 *)inp[p], inp[p], exp[p], g.Vh, nk, nullptr, 0, c.stream));
+            for (int p = 0; p < 2 && hops; p++) {
                 DslashParams P{};
                 P.in = inp[1 - p];
+                P.in_exp = exp[1 - p];
                 P.out = outp[p];
+                P.x = kind == DP_APPLY_FULL ? tmp[p] : nullptr;
                 P.links[0] = links[0];
                 P.links[1] = links[1];
                 P.hop = hopd;
                 P.g = g;
                 P.parity = p;
                 P.nrhs = nk;
-                int epi = EPI_HOP;
-                if (kind == DP_APPLY_FULL) {
-                    CUDA_OK(launch_clover_apply(cp, pr, c.stream));
-                    P.x = tmp[p];
-                    epi = EPI_XPY;
-                }
                 const Shape sh = c.launch_shape(g.Vh, pr, lf, nk);
-                CUDA_OK(launch_dslash(P, pr, lf, epi, sh.block, pr == 0 ? 1 : 2, c.stream));
+                CUDA_OK(launch_dslash(P, pr, lf, kind == DP_APPLY_FULL ? EPI_XPY : EPI_HOP, sh.block,
+                                      pr == 0 ? 1 : 2, c.stream));
             }
             CUDA_OK(launch_unpack_spinor(oe, oo, g, nk, pr, lex, c.stream));
             CUDA_OK(cudaMemcpyAsync(out, lex, nlex * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
             CUDA_OK(cudaStreamSynchronize(c.stream));
-            c.launches += 6;
+            c.launches += ex ? 8 : 6;
             return DP_OK;
         };
         ret = run();
@@ -792,6 +801,7 @@ dp_status dp_apply(dp_ctx *ctx, dp_field field, int kind, double M, const dp_pro
     c.release(te);
     c.release(to);
     c.release(hopd);
+    c.release(ex);
     cudaStreamSynchronize(c.stream);
     return ret;
 }
@@ -879,18 +889,44 @@ dp_status dp_dslash_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile 
                   "thread and 64, 96 or 128 threads per block");
         return DP_ERR_INVALID_ARG;
     }
+    // FP64: the integer kernel, with its input's conversion, where its scratch can be had
+    void *xw = nullptr;
+    int *xe = nullptr;
+    if (pr == 0 && f.unitary) {
+        xw = c.alloc((size_t)g.Vh * nrhs * 24 * 8);
+        xe = (int *)c.alloc((size_t)g.Vh * nrhs * sizeof(int));
+        if (xw && xe) {
+            P.in = xw;
+            P.in_exp = xe;
+        }
+    }
     cudaEvent_t a = c.get_event(), b = c.get_event();
-    CUDA_OK(cudaEventRecord(a, c.stream));
-    for (int k = 0; k < iters; k++)
-        CUDA_OK(launch_dslash(P, pr, lf, EPI_AINV, block, rpt, c.stream, stg));
-    CUDA_OK(cudaEventRecord(b, c.stream));
-    c.launches += iters;
+    auto run = [&]() -> dp_status {
+        CUDA_OK(cudaEventRecord(a, c.stream));
+        for (int k = 0; k < iters; k++) {
+            if (P.in_exp)
+                CUDA_OK(launch_to_fx((const double2 *)in, xw, xe, g.Vh, nrhs, nullptr, 0, c.stream));
+            CUDA_OK(launch_dslash(P, pr, lf, EPI_AINV, block, rpt, c.stream, stg));
+        }
+        CUDA_OK(cudaEventRecord(b, c.stream));
+        return DP_OK;
+    };
+    stt = run();
+    if (stt != DP_OK) {
+        c.release(xw);
+        c.release(xe);
+        c.release(hopd);
+        return stt;
+    }
+    c.launches += P.in_exp ? 2 * iters : iters;
     CUDA_OK(cudaEventSynchronize(b));
     float ms = 0;
     cudaEventElapsedTime(&ms, a, b);
     c.event_pool.push_back(a);
     c.event_pool.push_back(b);
     if (ms_out) *ms_out = ms / iters;
+    c.release(xw);
+    c.release(xe);
     c.release(hopd);
     return DP_OK;
 }

@@ -48,6 +48,11 @@ struct Op {
     int block = 128;
     int rpt = 1;     // RHS per thread of the Schur launches
     int stages = 0;  // shared-memory staging of the Schur launches (0: direct)
+    // FP64 in integer arithmetic (dslash_fx.cu) when non-NULL: an FP64-sized
+    // scratch vector for the converted input, and the exponents of it and of
+    // the intermediate vector ([Vh][nrhs] ints each)
+    void *xw = nullptr;
+    int *xe = nullptr, *te = nullptr;
 };
 
 struct InnerVecs {

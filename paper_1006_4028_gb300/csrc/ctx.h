@@ -37,6 +37,7 @@ struct CloverInv {
 struct Field {
     Geom g;
     int bc_t;
+    bool unitary = false;  // every link's rows have norm 1 (to 1e-3)
     double2 *l64[2] = {nullptr, nullptr};
     float2 *l32f[2] = {nullptr, nullptr};
     float4 *l32c[2] = {nullptr, nullptr};

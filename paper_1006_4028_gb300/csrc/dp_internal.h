@@ -84,6 +84,11 @@ struct DslashParams {
     // BiCGStab omega: f2 (one lane per RHS of a pair) [3][Vh][nrhs/2] holding
     // Re <out, x>, Im <out, x> and |out|^2 over the 12 components of a site
     void *dots;
+    // FP64 in integer arithmetic (dslash_fx.cu; unitary links): NULL, or `in`
+    // holds fx spinors with these exponents, per (site, RHS) [Vh][nrhs];
+    // out_exp (A^-1 epilogue): NULL, or write `out` as fx spinors too
+    const int *in_exp;
+    int *out_exp;
 };
 
 // ---- launch wrappers (dslash.cu) ----
@@ -102,6 +107,15 @@ cudaError_t launch_dslash(const DslashParams &p, int prec, int link_fmt, int epi
                           int rpt, cudaStream_t st, int stages = 0);
 bool dslash_rpt_ok(int nrhs, int rpt, int prec, int epi);
 bool dslash_staged_ok(int prec, int link_fmt, int epi, int rpt, int stages, int block);
+// the FP64 launches in integer arithmetic (dslash_fx.cu): p.in_exp != NULL.
+// An fx spinor field has the size and layout of an FP64 one, plus an int per
+// (site, RHS).  to_fx: FP64 -> fx (w == in: in place); sub_fx: out = a - t,
+// t fx; both for the RHS with mask[r * stride] != 0 (NULL: all)
+cudaError_t launch_dslash_fx(const DslashParams &p, int epi, cudaStream_t st);
+cudaError_t launch_to_fx(const double2 *in, void *w, int *ex, long long Vh, int n, const int *mask, int stride,
+                         cudaStream_t st);
+cudaError_t launch_sub_fx(const double2 *a, const void *t, const int *ex, double2 *out, long long Vh, int n,
+                          const int *mask, cudaStream_t st);
 // double-float Schur launches of the outer loop (dslash_df.cu): EPI_AINV
 // writes double-float, EPI_XMY_AINV reads x as double-float and writes FP64;
 // links LINK_DF_18, clover inverse float4 [36][Vh], hops float2 [grp][8][Lmax]
@@ -157,8 +171,10 @@ cudaError_t launch_clover_norm(BlasCtx &bc, const CloverApplyParams &p, double *
                                cudaStream_t st);
 
 // ---- field packing, sources, restore/contract (field.cu) ----
+// sets *not_unitary (device int, zeroed by the caller) if a row of any link
+// has a squared norm off 1 by more than 1e-3
 cudaError_t launch_pack_links(const double2 *lex, const Geom &g, double2 *l64[2], float2 *l32f[2],
-                              float4 *l32c[2], cudaStream_t st);
+                              float4 *l32c[2], int *not_unitary, cudaStream_t st);
 // lexicographic complex128 spinors [nrhs][V][12] <-> packed parity halves
 cudaError_t launch_pack_spinor(const double2 *lex, const Geom &g, int nrhs, int prec,
                                void *even, void *odd, cudaStream_t st);

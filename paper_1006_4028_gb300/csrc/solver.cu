@@ -57,8 +57,10 @@ struct Timed {
     ~Timed() { c->time_end(name, ev, st); }
 };
 
+// in_exp / out_exp: FP64 through dslash_fx.cu (see DslashParams)
 dp_status dslash(Ctx *c, const Op &op, int parity, int epi, const void *in, void *out,
-                 const void *x, const int *mask, int mask_stride, void *dots = nullptr)
+                 const void *x, const int *mask, int mask_stride, void *dots = nullptr,
+                 const int *in_exp = nullptr, int *out_exp = nullptr)
 {
     DslashParams P{};
     P.in = in;
@@ -70,6 +72,8 @@ dp_status dslash(Ctx *c, const Op &op, int parity, int epi, const void *in, void
     P.links[1] = op.links[1];
     for (int k = 0; k < kMaxGroups; k++) P.clov[k] = op.inv[parity][k];
     P.hop = op.hop;
+    P.in_exp = in_exp;
+    P.out_exp = out_exp;
     P.active = mask;
     P.active_stride = mask_stride;
     P.g = f.g;
@@ -103,16 +107,33 @@ void set_shape(Op &op, const Shape &sh)
 
 const int *state_mask(const RhsState *st) { return st ? &st[0].active : nullptr; }
 
+// FP64 vector -> fx form for the integer kernel
+dp_status to_fx(Ctx *c, const Op &op, const void *x, void *w, const int *mask, int mask_stride)
+{
+    cudaEvent_t ev;
+    c->time_begin("dslash_fp64", &ev, op.st);
+    CK(launch_to_fx(static_cast<const double2 *>(x), w, op.xe, op.f->g.Vh, op.nrhs, mask, mask_stride, op.st));
+    c->time_end("dslash_fp64", ev, op.st);
+    c->launches++;
+    return DP_OK;
+}
+
 // Schur operator on parity p (q = 1 - p):
-// y = Mhat x = x - A_pp^-1 D_pq A_qq^-1 D_qp x ; tmp (parity q) keeps A_qq^-1 D_qp x;
+// y = Mhat x = x - A_pp^-1 D_pq A_qq^-1 D_qp x ; tmp (parity q) keeps A_qq^-1 D_qp x
+// (as an fx vector with exponents op.te when op.xw is set);
 // dots (FP32, or NULL): the second launch also leaves the per-site sums of
 // <y, x> and |y|^2 there (DslashParams::dots)
 dp_status apply_mhat(Ctx *c, const Op &op, int p, const void *x, void *y, void *tmp,
                      const RhsState *mask, void *dots = nullptr)
 {
-    dp_status s = dslash(c, op, 1 - p, EPI_AINV, x, tmp, nullptr, state_mask(mask), kStateStride);
+    dp_status s = DP_OK;
+    if (op.xw) s = to_fx(c, op, x, op.xw, state_mask(mask), kStateStride);
+    if (s == DP_OK)
+        s = dslash(c, op, 1 - p, EPI_AINV, op.xw ? op.xw : x, tmp, nullptr, state_mask(mask), kStateStride, nullptr,
+                   op.xw ? op.xe : nullptr, op.xw ? op.te : nullptr);
     if (s != DP_OK) return s;
-    return dslash(c, op, p, EPI_XMY_AINV, tmp, y, x, state_mask(mask), kStateStride, dots);
+    return dslash(c, op, p, EPI_XMY_AINV, tmp, y, x, state_mask(mask), kStateStride, dots,
+                  op.xw ? op.te : nullptr);
 }
 
 // Adjoint Schur operator.  With the hopping part H(alpha_B) and the clover
@@ -139,9 +160,14 @@ dp_status apply_mhat_dag(Ctx *c, const Op &op, const Op &op_adj, int p, const vo
     CK(launch_clover_apply(cp, op.pr, op.st));
     c->time_end("clover_apply", ev, op.st);
     c->launches++;
-    dp_status s = dslash(c, op_adj, 1 - p, EPI_AINV, tmp_p, tmp_q, nullptr, state_mask(mask), kStateStride);
+    dp_status s = DP_OK;
+    if (op.xw) s = to_fx(c, op, tmp_p, tmp_p, state_mask(mask), kStateStride);
+    if (s == DP_OK)
+        s = dslash(c, op_adj, 1 - p, EPI_AINV, tmp_p, tmp_q, nullptr, state_mask(mask), kStateStride, nullptr,
+                   op.xw ? op.xe : nullptr, op.xw ? op.te : nullptr);
     if (s != DP_OK) return s;
-    return dslash(c, op_adj, p, EPI_XMY_G5, tmp_q, out, y, state_mask(mask), kStateStride);
+    return dslash(c, op_adj, p, EPI_XMY_G5, tmp_q, out, y, state_mask(mask), kStateStride, nullptr,
+                  op.xw ? op.te : nullptr);
 }
 
 }  // namespace
@@ -283,10 +309,24 @@ dp_status Batch::init()
     op64.links[1] = f->l64[1];
     op64.hop = hop64_d;
     op64.nrhs = n;
+    if (f->unitary) {
+        // the integer kernel's exponents; its converted input goes to to64,
+        // which holds a job's source only while the job is set up or finished.
+        // Without the memory (8 bytes per site and RHS to the vectors' 2000)
+        // the FP64 kernel serves.
+        const size_t ne = (size_t)Vh * n;
+        int *ex = (int *)get(2 * ne * sizeof(int));
+        if (ex) {
+            op64.xw = to64;
+            op64.xe = ex;
+            op64.te = ex + ne;
+        }
+    }
     set_shape(op64, c->launch_shape(Vh, 0, LINK_F64_18, n));
     opin = op64;
     opin.pr = ipr;
     opin.lf = ilf;
+    if (ipr != 0) opin.xw = nullptr;
     for (int p = 0; p < 2; p++) {
         dp_status e = field_links(c, *f, ilf, p, &opin.links[p]);
         if (e != DP_OK) return e;
@@ -512,7 +552,11 @@ dp_status Batch::admit(Job *j)
         cp.in = to64;
         cp.out = to64;
         CK(launch_clover_point(cp, g, slots_d, 1 - sp, st_));
-        s = dslash(c, op64, sp, EPI_AINV_XMY, to64, bh, y64, mask_d, 1);
+        // (t64 is free between rounds: the converted source goes there)
+        if (op64.xw) s = to_fx(c, op64, to64, t64, mask_d, 1);
+        if (s == DP_OK)
+            s = dslash(c, op64, sp, EPI_AINV_XMY, op64.xw ? t64 : to64, bh, y64, mask_d, 1, nullptr,
+                       op64.xw ? op64.xe : nullptr);
         if (s != DP_OK) return s;
     }
     CK(blas_zero_masked(x, Vh, n, mask_d, st_));
@@ -631,7 +675,7 @@ dp_status Batch::bicgstab(int max_iter, int *iters_done)
                 graph_max_iter = max_iter;
             }
             CK(cudaGraphLaunch(graph, st_));
-            c->launches += fused ? 8 : 10;
+            c->launches += fused ? 8 : opin.xw ? 12 : 10;
         }
         it++;
         if (it >= max_iter) break;
@@ -829,7 +873,7 @@ dp_status Batch::cgne(int max_iter, int *iters_done)
                 graph_max_iter = max_iter;
             }
             CK(cudaGraphLaunch(graph, st_));
-            c->launches += 10;
+            c->launches += opin.xw ? 12 : 10;
         }
         it++;
         if (it >= max_iter) break;
@@ -1161,7 +1205,10 @@ dp_status Batch::harvest(std::vector<Job *> &finished)
         cp.in = to64;
         cp.out = to64;
         CK(launch_clover_point(cp, g, slots_d, 1 - sp, st_));
-        CK(blas_sub64_masked(to64, t64, y64, Vh, n, mask_d, st_));
+        if (op64.xw && !xdf)
+            CK(launch_sub_fx(to64, t64, op64.te, y64, Vh, n, mask_d, st_));
+        else
+            CK(blas_sub64_masked(to64, t64, y64, Vh, n, mask_d, st_));
         // residual report: the full residual of (D'+M)S' = eta' is (A_pp rhat, 0)
         // with x_q rebuilt from x_p, so |A_pp rhat| / |eta'| (a few digits:
         // FP32 products, FP64 sums)
@@ -1545,6 +1592,14 @@ dp_status dp_schur_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile *
     const size_t tb = hop.size() * (pr == 0 ? sizeof(double) : sizeof(float));
     const size_t vb = (size_t)g.Vh * nrhs * 24 * (pr == 0 ? 8 : 4);
     void *hd = c.alloc(tb), *had = c.alloc(tb), *tp = c.alloc(vb), *tq = c.alloc(vb);
+    // FP64: exponents for the integer kernel (without them the FP64 kernel serves)
+    const size_t ne = (size_t)g.Vh * nrhs;
+    int *ex = pr == 0 && f.unitary ? (int *)c.alloc(2 * ne * sizeof(int)) : nullptr;
+    if (ex) {
+        op.xw = tp;
+        op.xe = ex;
+        op.te = ex + ne;
+    }
     auto run = [&]() -> dp_status {
         if (!hd || !had || !tp || !tq) {
             set_error("out of device memory (dp_schur_dev)");
@@ -1568,6 +1623,7 @@ dp_status dp_schur_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile *
     c.release(had);
     c.release(tp);
     c.release(tq);
+    c.release(ex);
     return s;
 }
 

@@ -98,9 +98,10 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_alpha(Cfg c, const void *rh,
             acc[1] += d.im;
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<2, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_alpha(st[r], acc[0], acc[1]);
+    double v[2];
+    const int r = threadIdx.x;
+    if (!reduce_last<2, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_alpha(st[r], v[0], v[1]);
 }
 
 // s = r - alpha v
@@ -134,15 +135,16 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_omega(Cfg c, const void *tv,
             acc[2] += snorm(t);
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<3, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_omega(st[r], acc[0], acc[1], acc[2]);
+    double v[3];
+    const int r = threadIdx.x;
+    if (!reduce_last<3, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_omega(st[r], v[0], v[1], v[2]);
 }
 
 // x += alpha p + omega s; r = s - omega t; rho' = <rhat, r>; |r|^2
 __global__ void __launch_bounds__(kMaxBlock) k_bicg_update(Cfg c, void *xv, void *rv, const void *pv, const void *sv,
                               const void *tv, const void *rh, long long Vh, int nrhs,
-                              RhsState *st, int max_iter, double *partials, unsigned int *counter)
+                              RhsState *st, int max_iter, double *partials, unsigned int *counter, int *n_active)
 {
     double acc[3] = {0, 0, 0};
     {
@@ -166,14 +168,16 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_update(Cfg c, void *xv, void
             acc[2] += snorm(sx);
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<3, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_update(st[r], acc[0], acc[1], acc[2], max_iter);
+    double v[3];
+    const int r = threadIdx.x;
+    if (!reduce_last<3, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_update(st[r], v[0], v[1], v[2], max_iter);
+    count_active(st, nrhs, n_active);
 }
 
 // inner init: r = b, rhat = r (b may alias rhat); rho = |r|^2, tol2 *= |r|^2
 __global__ void __launch_bounds__(kMaxBlock) k_bicg_init(Cfg c, const void *bv, void *rv, void *rh, long long Vh, int nrhs,
-                            RhsState *st, double *partials, unsigned int *counter)
+                            RhsState *st, double *partials, unsigned int *counter, int *n_active)
 {
     double acc[1] = {0};
     {
@@ -186,9 +190,11 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_init(Cfg c, const void *bv, 
             acc[0] += snorm(b);
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_init(st[r], acc[0]);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_init(st[r], v[0]);
+    count_active(st, nrhs, n_active);
 }
 
 // ---- CGNE on the normal equations (real per-RHS scalars) ----
@@ -202,9 +208,10 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_gamma(Cfg c, const void *zv, l
     {
         SITE_LOOP acc[0] += snorm(ld(zv, cs, s * n + r));
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_cg_gamma(st[r], acc[0], first);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_cg_gamma(st[r], v[0], first);
 }
 
 // p = z + beta p
@@ -235,16 +242,17 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_alpha(Cfg c, const void *wv, l
     {
         SITE_LOOP acc[0] += snorm(ld(wv, cs, s * n + r));
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_cg_alpha(st[r], acc[0]);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_cg_alpha(st[r], v[0]);
 }
 
 // x += alpha p, r -= alpha w, |r|^2
 __global__ void __launch_bounds__(kMaxBlock) k_cg_update(Cfg c, void *xv, void *rv, const void *pv,
                                                          const void *wv, long long Vh, int nrhs,
                                                          RhsState *st, int max_iter, double *partials,
-                                                         unsigned int *counter)
+                                                         unsigned int *counter, int *n_active)
 {
     double acc[1] = {0};
     {
@@ -271,9 +279,11 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_update(Cfg c, void *xv, void *
             acc[0] += snorm(rr);
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    finish_cg_update(st[r], acc[0], max_iter);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs) finish_cg_update(st[r], v[0], max_iter);
+    count_active(st, nrhs, n_active);
 }
 
 // FP64 outer residual r = b - y and |r|^2; an RHS flagged `fresh` (x = 0)
@@ -281,7 +291,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_update(Cfg c, void *xv, void *
 // absolute threshold r_target^2 |b|^2
 __global__ void __launch_bounds__(kMaxBlock) k_residual64(Cfg c, const double2 *b, const double2 *y, double2 *rv,
                              long long Vh, int nrhs, RhsState *st, const int *mask,
-                             double *partials, unsigned int *counter)
+                             double *partials, unsigned int *counter, int *n_active)
 {
     double acc[2] = {0, 0};
     const bool use = !mask || mask[threadIdx.x % nrhs];
@@ -302,24 +312,27 @@ __global__ void __launch_bounds__(kMaxBlock) k_residual64(Cfg c, const double2 *
             acc[0] += snorm(bb);
         }
     }
-    const int r = threadIdx.x % nrhs;
-    if (!reduce_last<2, 1>(acc, c, partials, counter, nrhs)) return;
-    RhsState &S = st[r];
-    if (!S.active || !use) return;
-    if (S.fresh) {
-        S.bb = acc[1];
-        S.tol2 = S.tol2 * acc[1];
-        S.fresh = 0;
+    double v[2];
+    const int r = threadIdx.x;
+    if (!reduce_last<2, 1>(acc, c, partials, counter, nrhs, v)) return;
+    if (r < nrhs && st[r].active && use) {
+        RhsState &S = st[r];
+        if (S.fresh) {
+            S.bb = v[1];
+            S.tol2 = S.tol2 * v[1];
+            S.fresh = 0;
+        }
+        S.rr = v[0];
+        S.scale = sqrt(v[0]);
+        if (!isfinite(v[0])) {
+            S.status = 3;
+            S.active = 0;
+        } else if (!S.refine && v[0] <= S.tol2) {  // a refined RHS stops on its slices
+            S.status = 1;
+            S.active = 0;
+        }
     }
-    S.rr = acc[0];
-    S.scale = sqrt(acc[0]);
-    if (!isfinite(acc[0])) {
-        S.status = 3;
-        S.active = 0;
-    } else if (!S.refine && acc[0] <= S.tol2) {  // a refined RHS stops on its slices
-        S.status = 1;
-        S.active = 0;
-    }
+    count_active(st, nrhs, n_active);
 }
 
 __global__ void __launch_bounds__(kMaxBlock) k_norm2(Cfg c, const double2 *v, long long Vh, int nrhs, double *out,
@@ -331,8 +344,9 @@ __global__ void __launch_bounds__(kMaxBlock) k_norm2(Cfg c, const double2 *v, lo
     const long long cs = Vh * n;
     for (long long s = (long long)blockIdx.x * c.lanes + lane; s < Vh; s += (long long)gridDim.x * c.lanes)
         acc[0] += snorm(ld(v, cs, s * n + r));
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    out[r] = acc[0];
+    double tot[1];
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, tot)) return;
+    if ((int)threadIdx.x < nrhs) out[threadIdx.x] = tot[0];
 }
 
 __global__ void __launch_bounds__(kMaxBlock) k_diff_norm2(Cfg c, const double2 *a, const double2 *b, long long Vh, int nrhs,
@@ -349,15 +363,9 @@ __global__ void __launch_bounds__(kMaxBlock) k_diff_norm2(Cfg c, const double2 *
         for (int k = 0; k < 12; k++) x.c[k] = x.c[k] - y.c[k];
         acc[0] += snorm(x);
     }
-    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs)) return;
-    out[r] = acc[0];
-}
-
-__global__ void k_count_active(const RhsState *st, int n, int *n_active)
-{
-    int c = 0;
-    for (int r = 0; r < n; r++) c += st[r].active ? 1 : 0;
-    *n_active = c;
+    double tot[1];
+    if (!reduce_last<1, 1>(acc, c, partials, counter, nrhs, tot)) return;
+    if ((int)threadIdx.x < nrhs) out[threadIdx.x] = tot[0];
 }
 
 // inner state from the outer one: same active set.  The outer threshold is
@@ -447,12 +455,6 @@ inline unsigned blocks_for(long long n, int b) { return (unsigned)((n + b - 1) /
 
 cudaError_t blas_zero(void *v, size_t bytes, cudaStream_t s) { return cudaMemsetAsync(v, 0, bytes, s); }
 
-cudaError_t blas_count_active(BlasCtx &bc, const RhsState *st, int nrhs, cudaStream_t s)
-{
-    k_count_active<<<1, 1, 0, s>>>(st, nrhs, bc.n_active);
-    return cudaGetLastError();
-}
-
 cudaError_t blas_bicg_init(BlasCtx &bc, int prec, const void *b, void *r, void *rhat, void *p,
                            void *v, void *x, long long Vh, int nrhs, RhsState *st, double tol,
                            cudaStream_t s)
@@ -463,15 +465,12 @@ cudaError_t blas_bicg_init(BlasCtx &bc, int prec, const void *b, void *r, void *
     cudaMemsetAsync(v, 0, bytes, s);
     cudaMemsetAsync(x, 0, bytes, s);
     if (prec != 0) {
-        cudaError_t e = blas32_init(bc, b, r, rhat, Vh, nrhs, st, s);
-        if (e != cudaSuccess) return e;
+        return blas32_init(bc, b, r, rhat, Vh, nrhs, st, s);
     } else {
         const Cfg c = cfg_wave(bc, k_bicg_init, Vh, nrhs);
-        k_bicg_init<<<c.grid, c.block, 0, s>>>(c, b, r, rhat, Vh, nrhs, st, bc.partials, bc.counter);
+        k_bicg_init<<<c.grid, c.block, 0, s>>>(c, b, r, rhat, Vh, nrhs, st, bc.partials, bc.counter, bc.n_active);
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+    return cudaGetLastError();
 }
 
 cudaError_t blas_bicg_p(BlasCtx &bc, int prec, const void *r, void *p, const void *v,
@@ -520,11 +519,10 @@ cudaError_t blas_bicg_update(BlasCtx &bc, int prec, void *x, void *r, const void
     } else {
         const Cfg c = cfg_wave(bc, k_bicg_update, Vh, nrhs);
         k_bicg_update<<<c.grid, c.block, 0, s>>>(c, x, r, p, sv, t, rhat, Vh, nrhs, st, max_iter,
-                                                 bc.partials, bc.counter);
+                                                 bc.partials, bc.counter, bc.n_active);
         e = cudaGetLastError();
     }
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+    return e;
 }
 
 cudaError_t blas_cg_gamma(BlasCtx &bc, int prec, const void *z, long long Vh, int nrhs,
@@ -563,21 +561,18 @@ cudaError_t blas_cg_update(BlasCtx &bc, int prec, void *x, void *r, const void *
     } else {
         const Cfg c = cfg_wave(bc, k_cg_update, Vh, nrhs);
         k_cg_update<<<c.grid, c.block, 0, s>>>(c, x, r, p, w, Vh, nrhs, st, max_iter, bc.partials,
-                                               bc.counter);
+                                               bc.counter, bc.n_active);
         e = cudaGetLastError();
     }
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+    return e;
 }
 
 cudaError_t blas_residual64(BlasCtx &bc, const double2 *b, const double2 *y, double2 *r,
                             long long Vh, int nrhs, RhsState *st, const int *mask, cudaStream_t s)
 {
     const Cfg c = cfg_wave(bc, k_residual64, Vh, nrhs);
-    k_residual64<<<c.grid, c.block, 0, s>>>(c, b, y, r, Vh, nrhs, st, mask, bc.partials, bc.counter);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+    k_residual64<<<c.grid, c.block, 0, s>>>(c, b, y, r, Vh, nrhs, st, mask, bc.partials, bc.counter, bc.n_active);
+    return cudaGetLastError();
 }
 
 cudaError_t blas_norm2(BlasCtx &bc, int prec, const void *v, long long Vh, int nrhs,

@@ -4,7 +4,7 @@
 // products are summed in FP32 over the sites one thread visits (24 terms a
 // site, a few tens of sites: one packed f32x2 add per site and value, where
 // an FP64 add per site would run on GB300's 1/64-rate FP64 pipe) and across
-// threads and blocks in FP64 per RHS; the reductions and the scalar
+// threads and blocks on 64-bit integers per RHS; the reductions and the scalar
 // recurrences (those the FP64 kernels share, and the shadow-form BiCGStab's
 // own) are in reduce.cuh, so every decision stays per RHS.
 //
@@ -46,10 +46,7 @@ __device__ __forceinline__ void st1(void *base, long long cs, long long me, int 
 }
 
 // per-lane complex scalar from the two RHS states
-__device__ __forceinline__ C2 lanes(double2 a0, double2 a1)
-{
-    return {pk((float)a0.x, (float)a1.x), pk((float)a0.y, (float)a1.y)};
-}
+__device__ __forceinline__ C2 lanes(float2 a0, float2 a1) { return {pk(a0.x, a1.x), pk(a0.y, a1.y)}; }
 __device__ __forceinline__ C2 neg(C2 a) { return {fneg2(a.re), fneg2(a.im)}; }
 
 // <a, b> per lane over one site, FP32
@@ -76,27 +73,31 @@ __device__ __forceinline__ f2 pnorm(const P12 &a)
     return s;
 }
 
-// add the two lanes of an f2 into FP64 accumulators, only for active lanes
-__device__ __forceinline__ void add_lanes(double &d0, double &d1, f2 v, bool a0, bool a1)
+// the two lanes of a thread's sum, zero for an inactive RHS
+__device__ __forceinline__ void set_lanes(float &d0, float &d1, f2 v, bool a0, bool a1)
 {
     float l0, l1;
     upk(v, l0, l1);
-    if (a0) d0 += (double)l0;
-    if (a1) d1 += (double)l1;
+    d0 = a0 ? l0 : 0.f;
+    d1 = a1 ? l1 : 0.f;
 }
 
-#define PAIR_LOOP                                                              \
+#define PAIR_VARS                                                              \
     const int P = nrhs / 2;                                                    \
     const int q = threadIdx.x % P, lane = threadIdx.x / P;                     \
     const long long cs = Vh * P;                                               \
-    const bool a0 = st[2 * q].active != 0, a1 = st[2 * q + 1].active != 0;     \
+    const bool a0 = st[2 * q].active != 0, a1 = st[2 * q + 1].active != 0
+#define PAIR_FOR                                                               \
     for (long long s = (long long)blockIdx.x * c.lanes + lane; (a0 || a1) && s < Vh; \
          s += (long long)gridDim.x * c.lanes)
+#define PAIR_LOOP                                                              \
+    PAIR_VARS;                                                                 \
+    PAIR_FOR
 
 __global__ void __launch_bounds__(kMaxBlock) k32_alpha(Cfg c, const void *rh, const void *vv, long long Vh, int nrhs,
-                          RhsState *st, double *partials, unsigned int *counter)
+                          RhsState *st, double *partials, unsigned int *counter, int *n_active)
 {
-    double acc[4] = {0, 0, 0, 0};  // lane 0: re, im; lane 1: re, im
+    float acc[4];  // RHS 2q: re, im; 2q + 1: re, im
     {
         f2 sum0 = 0ull, sum1 = 0ull;
         PAIR_LOOP
@@ -106,13 +107,14 @@ __global__ void __launch_bounds__(kMaxBlock) k32_alpha(Cfg c, const void *rh, co
             sum0 = fadd2(sum0, d.re);
             sum1 = fadd2(sum1, d.im);
         }
-        add_lanes(acc[0], acc[2], sum0, a0, a1);
-        add_lanes(acc[1], acc[3], sum1, a0, a1);
+        set_lanes(acc[0], acc[2], sum0, a0, a1);
+        set_lanes(acc[1], acc[3], sum1, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<2, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_alpha(st[2 * q], acc[0], acc[1]);
-    finish_alpha(st[2 * q + 1], acc[2], acc[3]);
+    double v[2];
+    const int r = threadIdx.x;
+    if (!reduce_last<2, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_alpha(st[r], v[0], v[1]);
+    count_active(st, nrhs, n_active);
 }
 
 // keep the lanes of `old` whose RHS is inactive
@@ -120,9 +122,9 @@ __device__ __forceinline__ f2 blend(f2 nw, f2 old, f2 m) { return (nw & m) | (ol
 
 __global__ void __launch_bounds__(kMaxBlock) k32_init(Cfg c, const void *bv, void *rv, void *rh, void *pv,
                                                       long long Vh, int nrhs, RhsState *st,
-                                                      double *partials, unsigned int *counter)
+                                                      double *partials, unsigned int *counter, int *n_active)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         f2 sum0 = 0ull;
         PAIR_LOOP
@@ -134,12 +136,13 @@ __global__ void __launch_bounds__(kMaxBlock) k32_init(Cfg c, const void *bv, voi
             if (pv) stp(pv, cs, me, b);
             sum0 = fadd2(sum0, pnorm(b));
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_init(st[2 * q], acc[0]);
-    finish_init(st[2 * q + 1], acc[1]);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_init(st[r], v[0]);
+    count_active(st, nrhs, n_active);
 }
 
 // ---- BiCGStab with the shadow image rhat' = Mhat^dag rhat ----
@@ -155,12 +158,10 @@ __global__ void __launch_bounds__(kMaxBlock) k32_s_dots(Cfg c, const void *rv, c
                                                         long long Vh, int nrhs, RhsState *st,
                                                         double *partials, unsigned int *counter)
 {
-    double acc[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) acc[k] = 0;
+    float acc[8];
     {
         const int qq = threadIdx.x % (nrhs / 2);
-        const C2 mal = neg(lanes(st[2 * qq].alpha, st[2 * qq + 1].alpha));
+        const C2 mal = neg(lanes(st[2 * qq].alpha_f, st[2 * qq + 1].alpha_f));
         f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull, sum3 = 0ull;
         PAIR_LOOP
         {
@@ -188,53 +189,56 @@ __global__ void __launch_bounds__(kMaxBlock) k32_s_dots(Cfg c, const void *rv, c
             sum2 = fadd2(sum2, rtr);
             sum3 = fadd2(sum3, rti);
         }
-        add_lanes(acc[0], acc[4], sum0, a0, a1);
-        add_lanes(acc[1], acc[5], sum1, a0, a1);
-        add_lanes(acc[2], acc[6], sum2, a0, a1);
-        add_lanes(acc[3], acc[7], sum3, a0, a1);
+        set_lanes(acc[0], acc[4], sum0, a0, a1);
+        set_lanes(acc[1], acc[5], sum1, a0, a1);
+        set_lanes(acc[2], acc[6], sum2, a0, a1);
+        set_lanes(acc[3], acc[7], sum3, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<4, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_s_dots(st[2 * q], acc[0], acc[1], acc[2], acc[3]);
-    finish_s_dots(st[2 * q + 1], acc[4], acc[5], acc[6], acc[7]);
+    double v[4];
+    const int r = threadIdx.x;
+    if (!reduce_last<4, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_s_dots(st[r], v[0], v[1], v[2], v[3]);
 }
 
 __global__ void __launch_bounds__(kMaxBlock) k32_omega_dots(Cfg c, const void *dots, long long Vh,
                                                             int nrhs, RhsState *st,
                                                             double *partials, unsigned int *counter)
 {
-    double acc[6] = {0, 0, 0, 0, 0, 0};
+    float acc[6];
     {
         const f2 *d = static_cast<const f2 *>(dots);
         f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull;
-        PAIR_LOOP
+        PAIR_VARS;
+        // (three loads an item: four items' in flight)
+#pragma unroll 4
+        PAIR_FOR
         {
             const long long me = s * P + q;
             sum0 = fadd2(sum0, __ldg(d + me));
             sum1 = fadd2(sum1, __ldg(d + cs + me));
             sum2 = fadd2(sum2, __ldg(d + 2 * cs + me));
         }
-        add_lanes(acc[0], acc[3], sum0, a0, a1);
-        add_lanes(acc[1], acc[4], sum1, a0, a1);
-        add_lanes(acc[2], acc[5], sum2, a0, a1);
+        set_lanes(acc[0], acc[3], sum0, a0, a1);
+        set_lanes(acc[1], acc[4], sum1, a0, a1);
+        set_lanes(acc[2], acc[5], sum2, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<3, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_omega_shadow(st[2 * q], acc[0], acc[1], acc[2]);
-    finish_omega_shadow(st[2 * q + 1], acc[3], acc[4], acc[5]);
+    double v[3];
+    const int r = threadIdx.x;
+    if (!reduce_last<3, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_omega_shadow(st[r], v[0], v[1], v[2]);
 }
 
 __global__ void __launch_bounds__(kMaxBlock)
 k32_update_pa(Cfg c, void *xv, void *rv, void *pv, const void *sv, const void *tv, const void *vv,
               const void *rh2, long long Vh, int nrhs, RhsState *st, int max_iter,
-              double *partials, unsigned int *counter)
+              double *partials, unsigned int *counter, int *n_active)
 {
-    double acc[6] = {0, 0, 0, 0, 0, 0};
+    float acc[6];
     {
         const int qq = threadIdx.x % (nrhs / 2);
-        const C2 al = lanes(st[2 * qq].alpha, st[2 * qq + 1].alpha);
-        const C2 om = lanes(st[2 * qq].omega, st[2 * qq + 1].omega);
-        const C2 be = lanes(st[2 * qq].beta, st[2 * qq + 1].beta);
+        const C2 al = lanes(st[2 * qq].alpha_f, st[2 * qq + 1].alpha_f);
+        const C2 om = lanes(st[2 * qq].omega_f, st[2 * qq + 1].omega_f);
+        const C2 be = lanes(st[2 * qq].beta_f, st[2 * qq + 1].beta_f);
         const C2 mom = neg(om);
         f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull;
         PAIR_LOOP
@@ -266,29 +270,31 @@ k32_update_pa(Cfg c, void *xv, void *rv, void *pv, const void *sv, const void *t
             sum1 = fadd2(sum1, rpr);
             sum2 = fadd2(sum2, rpi);
         }
-        add_lanes(acc[0], acc[3], sum0, a0, a1);
-        add_lanes(acc[1], acc[4], sum1, a0, a1);
-        add_lanes(acc[2], acc[5], sum2, a0, a1);
+        set_lanes(acc[0], acc[3], sum0, a0, a1);
+        set_lanes(acc[1], acc[4], sum1, a0, a1);
+        set_lanes(acc[2], acc[5], sum2, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<3, 2>(acc, c, partials, counter, nrhs / 2)) return;
+    double v[3];
+    const int r = threadIdx.x;
+    if (!reduce_last<3, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
     // convergence on |r|^2, then the next alpha = rho' / <rhat', p> for the
     // RHS still iterating
-    finish_update_rr(st[2 * q], acc[0], max_iter);
-    finish_alpha(st[2 * q], acc[1], acc[2]);
-    finish_update_rr(st[2 * q + 1], acc[3], max_iter);
-    finish_alpha(st[2 * q + 1], acc[4], acc[5]);
+    if (r < nrhs) {
+        finish_update_rr(st[r], v[0], max_iter);
+        finish_alpha(st[r], v[1], v[2]);
+    }
+    count_active(st, nrhs, n_active);
 }
 
 // ---- CGNE on the normal equations: real per-RHS scalars, per lane ----
 
-__device__ __forceinline__ f2 lanes_re(double a0, double a1) { return pk((float)a0, (float)a1); }
+__device__ __forceinline__ f2 lanes_re(float a0, float a1) { return pk(a0, a1); }
 
 __global__ void __launch_bounds__(kMaxBlock)
 k32_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs, RhsState *st, int first,
              double *partials, unsigned int *counter)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         f2 sum0 = 0ull;
         PAIR_LOOP
@@ -303,12 +309,12 @@ k32_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs, RhsState *st, int fi
             }
             sum0 = fadd2(sum0, nn);
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_cg_gamma(st[2 * q], acc[0], first);
-    finish_cg_gamma(st[2 * q + 1], acc[1], first);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_cg_gamma(st[r], v[0], first);
 }
 
 // p = z + beta p
@@ -316,7 +322,7 @@ __global__ void __launch_bounds__(kMaxBlock)
 k32_cg_p(Cfg c, const void *zv, void *pv, long long Vh, int nrhs, const RhsState *st)
 {
     const int qq = threadIdx.x % (nrhs / 2);
-    const f2 be = lanes_re(st[2 * qq].beta.x, st[2 * qq + 1].beta.x);
+    const f2 be = lanes_re(st[2 * qq].beta_f.x, st[2 * qq + 1].beta_f.x);
     PAIR_LOOP
     {
         const long long me = s * P + q;
@@ -336,7 +342,7 @@ __global__ void __launch_bounds__(kMaxBlock)
 k32_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs, RhsState *st, double *partials,
              unsigned int *counter)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         f2 sum0 = 0ull;
         PAIR_LOOP
@@ -351,23 +357,23 @@ k32_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs, RhsState *st, double
             }
             sum0 = fadd2(sum0, nn);
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_cg_alpha(st[2 * q], acc[0]);
-    finish_cg_alpha(st[2 * q + 1], acc[1]);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_cg_alpha(st[r], v[0]);
 }
 
 // x += alpha p (active lanes only), r -= alpha w, |r|^2
 __global__ void __launch_bounds__(kMaxBlock)
 k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long long Vh, int nrhs,
-              RhsState *st, int max_iter, double *partials, unsigned int *counter)
+              RhsState *st, int max_iter, double *partials, unsigned int *counter, int *n_active)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         const int qq = threadIdx.x % (nrhs / 2);
-        const f2 al = lanes_re(st[2 * qq].alpha.x, st[2 * qq + 1].alpha.x);
+        const f2 al = lanes_re(st[2 * qq].alpha_f.x, st[2 * qq + 1].alpha_f.x);
         const f2 mal = fneg2(al);
         f2 sum0 = 0ull;
         PAIR_LOOP
@@ -392,12 +398,13 @@ k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long lo
             }
             sum0 = fadd2(sum0, nn);
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_cg_update(st[2 * q], acc[0], max_iter);
-    finish_cg_update(st[2 * q + 1], acc[1], max_iter);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_cg_update(st[r], v[0], max_iter);
+    count_active(st, nrhs, n_active);
 }
 
 // ---- GCR (the Krylov part of SAP+GCR): per-RHS dot products into device
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(kMaxBlock)
 k32_dotv(Cfg c, const void *av, const void *bv, long long Vh, int nrhs, const RhsState *st,
          double2 *out, double *partials, unsigned int *counter)
 {
-    double acc[4] = {0, 0, 0, 0};
+    float acc[4];
     {
         f2 sum0 = 0ull, sum1 = 0ull;
         PAIR_LOOP
@@ -426,13 +433,13 @@ k32_dotv(Cfg c, const void *av, const void *bv, long long Vh, int nrhs, const Rh
             sum0 = fadd2(sum0, re);
             sum1 = fadd2(sum1, im);
         }
-        add_lanes(acc[0], acc[2], sum0, a0, a1);
-        add_lanes(acc[1], acc[3], sum1, a0, a1);
+        set_lanes(acc[0], acc[2], sum0, a0, a1);
+        set_lanes(acc[1], acc[3], sum1, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<2, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    out[2 * q] = make_double2(acc[0], acc[1]);
-    out[2 * q + 1] = make_double2(acc[2], acc[3]);
+    double v[2];
+    const int r = threadIdx.x;
+    if (!reduce_last<2, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) out[r] = make_double2(v[0], v[1]);
 }
 
 // out[r] = |a|^2 per RHS
@@ -440,7 +447,7 @@ __global__ void __launch_bounds__(kMaxBlock)
 k32_norm2v(Cfg c, const void *av, long long Vh, int nrhs, const RhsState *st, double *out,
            double *partials, unsigned int *counter)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         f2 sum0 = 0ull;
         PAIR_LOOP
@@ -455,12 +462,12 @@ k32_norm2v(Cfg c, const void *av, long long Vh, int nrhs, const RhsState *st, do
             }
             sum0 = fadd2(sum0, nn);
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    out[2 * q] = acc[0];
-    out[2 * q + 1] = acc[1];
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) out[r] = v[0];
 }
 
 __device__ __forceinline__ C2 coef_lanes(const double2 *cf, int q, double sign)
@@ -513,9 +520,9 @@ k32_normalise(Cfg c, void *wv, void *zv, long long Vh, int nrhs, const RhsState 
 __global__ void __launch_bounds__(kMaxBlock)
 k32_gcr_update(Cfg c, void *xv, void *rv, const void *zv, const void *wv, long long Vh, int nrhs,
                RhsState *st, const double2 *cf, int max_iter, double *partials,
-               unsigned int *counter)
+               unsigned int *counter, int *n_active)
 {
-    double acc[2] = {0, 0};
+    float acc[2];
     {
         const int qq = threadIdx.x % (nrhs / 2);
         const C2 a = coef_lanes(cf, qq, 1.0), ma = coef_lanes(cf, qq, -1.0);
@@ -539,12 +546,13 @@ k32_gcr_update(Cfg c, void *xv, void *rv, const void *zv, const void *wv, long l
             }
             sum0 = fadd2(sum0, nn);
         }
-        add_lanes(acc[0], acc[1], sum0, a0, a1);
+        set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
-    const int q = threadIdx.x % (nrhs / 2);
-    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2)) return;
-    finish_cg_update(st[2 * q], acc[0], max_iter);
-    finish_cg_update(st[2 * q + 1], acc[1], max_iter);
+    double v[1];
+    const int r = threadIdx.x;
+    if (!reduce_last<1, 2>(acc, c, partials, counter, nrhs / 2, v)) return;
+    if (r < nrhs) finish_cg_update(st[r], v[0], max_iter);
+    count_active(st, nrhs, n_active);
 }
 
 // out = a - b (every pair)
@@ -617,7 +625,7 @@ cudaError_t blas32_init(BlasCtx &bc, const void *b, void *r, void *rh, long long
 {
     if (nrhs % 2) return cudaErrorInvalidValue;
     const Cfg c = cfg_wave(bc, k32_init, Vh, nrhs / 2);
-    k32_init<<<c.grid, c.block, 0, s>>>(c, b, r, rh, p, Vh, nrhs, st, bc.partials, bc.counter);
+    k32_init<<<c.grid, c.block, 0, s>>>(c, b, r, rh, p, Vh, nrhs, st, bc.partials, bc.counter, bc.n_active);
     return cudaGetLastError();
 }
 
@@ -646,10 +654,8 @@ cudaError_t blas32_update_pa(BlasCtx &bc, void *x, void *r, void *p, const void 
     if (nrhs % 2) return cudaErrorInvalidValue;
     const Cfg c = cfg_wave(bc, k32_update_pa, Vh, nrhs / 2);
     k32_update_pa<<<c.grid, c.block, 0, s>>>(c, x, r, p, sv, t, v, rh2, Vh, nrhs, st, max_iter,
-                                             bc.partials, bc.counter);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+                                             bc.partials, bc.counter, bc.n_active);
+    return cudaGetLastError();
 }
 
 cudaError_t blas32_alpha(BlasCtx &bc, const void *rh, const void *v, long long Vh, int nrhs,
@@ -657,7 +663,7 @@ cudaError_t blas32_alpha(BlasCtx &bc, const void *rh, const void *v, long long V
 {
     if (nrhs % 2) return cudaErrorInvalidValue;
     const Cfg c = cfg_wave(bc, k32_alpha, Vh, nrhs / 2);
-    k32_alpha<<<c.grid, c.block, 0, s>>>(c, rh, v, Vh, nrhs, st, bc.partials, bc.counter);
+    k32_alpha<<<c.grid, c.block, 0, s>>>(c, rh, v, Vh, nrhs, st, bc.partials, bc.counter, bc.n_active);
     return cudaGetLastError();
 }
 
@@ -694,7 +700,7 @@ cudaError_t blas32_cg_update(BlasCtx &bc, void *x, void *r, const void *p, const
     if (nrhs % 2) return cudaErrorInvalidValue;
     const Cfg c = cfg_wave(bc, k32_cg_update, Vh, nrhs / 2);
     k32_cg_update<<<c.grid, c.block, 0, s>>>(c, x, r, p, w, Vh, nrhs, st, max_iter, bc.partials,
-                                             bc.counter);
+                                             bc.counter, bc.n_active);
     return cudaGetLastError();
 }
 
@@ -741,10 +747,8 @@ cudaError_t blas32_gcr_update(BlasCtx &bc, void *x, void *r, const void *z, cons
     if (nrhs % 2) return cudaErrorInvalidValue;
     const Cfg c = cfg_wave(bc, k32_gcr_update, Vh, nrhs / 2);
     k32_gcr_update<<<c.grid, c.block, 0, s>>>(c, x, r, z, w, Vh, nrhs, st, cf, max_iter, bc.partials,
-                                              bc.counter);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return blas_count_active(bc, st, nrhs, s);
+                                              bc.counter, bc.n_active);
+    return cudaGetLastError();
 }
 
 cudaError_t blas32_xmy(const void *a, const void *b, void *out, long long Vh, int nrhs, cudaStream_t s)

@@ -377,8 +377,9 @@ __global__ void __launch_bounds__(kMaxBlock)
         for (int k = 0; k < 12; k++) ss = fmx(w[k].re, w[k].re, fmx(w[k].im, w[k].im, ss));
         acc[0] += (double)ss;
     }
-    if (!reduce_last<1, 1>(acc, c, partials, counter, n)) return;
-    out[r] = acc[0];
+    double tot[1];
+    if (!reduce_last<1, 1>(acc, c, partials, counter, n, tot)) return;
+    if ((int)threadIdx.x < n) out[threadIdx.x] = tot[0];
 }
 
 // FP64 [36 double2][Vh] -> FP32 [18 float4][Vh], same order of the 72 reals

@@ -220,6 +220,9 @@ struct RhsState {        // per RHS, device resident
     int refine;           // FP64 outer loop: per-slice refinement (the inner solve runs in
                           // another profile's metric; the global test does not stop it)
     double2 rs, rt;       // FP32 BiCGStab: <rhat, s> and <rhat', s> = <rhat, Mhat s>
+    // alpha, omega, beta as the FP32 kernels take them (converted once, by the
+    // thread that sets them: a conversion costs a warp 64 cycles)
+    float2 alpha_f, omega_f, beta_f;
 };
 
 constexpr int kRedWidth = 8;  // values per RHS in a block's reduction partials
@@ -227,7 +230,7 @@ constexpr int kRedWidth = 8;  // values per RHS in a block's reduction partials
 struct BlasCtx {
     double *partials;     // [max_blocks][kMaxRhs][kRedWidth]
     unsigned int *counter;
-    int *n_active;        // device counter of active RHS
+    int *n_active;        // active RHS after the last init / update / residual pass
     int blocks;
 };
 
@@ -396,7 +399,5 @@ cudaError_t blas_acc64(double2 *x64, const double2 *e64, long long Vh, int nrhs,
 // per-RHS |a - b|^2 (FP64) into out_dev[nrhs]
 cudaError_t blas_diff_norm2(BlasCtx &bc, const double2 *a, const double2 *b, long long Vh,
                             int nrhs, double *out_dev, cudaStream_t s);
-// count active RHS into bc.n_active
-cudaError_t blas_count_active(BlasCtx &bc, const RhsState *st, int nrhs, cudaStream_t s);
 
 }  // namespace dp

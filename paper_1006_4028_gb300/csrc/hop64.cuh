@@ -72,6 +72,13 @@ __device__ __forceinline__ void accumulate(Cx<R> acc[12], const Cx<R> uh[6], R c
 // int64) that stand for all components zero and for raw doubles in place of W
 constexpr int kFxZero = -1, kFxRaw = -2;
 
+// W 2^k as FP64; the exponents of fx spinors keep every non-zero result normal
+__device__ __forceinline__ double fx_value(long long w, int k)
+{
+    const double d = (double)w;
+    return w ? __hiloint2double(__double2hiint(d) + k * (1 << 20), __double2loint(d)) : 0.0;
+}
+
 // one fx spinor as FP64
 __device__ __forceinline__ void load_fx(const longlong2 *b, long long cs, int e, Cx<double> s[12])
 {
@@ -81,7 +88,7 @@ __device__ __forceinline__ void load_fx(const longlong2 *b, long long cs, int e,
         if (e == kFxRaw)
             s[k] = {__longlong_as_double(w.x), __longlong_as_double(w.y)};
         else
-            s[k] = {scalbn(__ll2double_rn(w.x), e - 1023 - 59), scalbn(__ll2double_rn(w.y), e - 1023 - 59)};
+            s[k] = {fx_value(w.x, e - 1023 - 59), fx_value(w.y, e - 1023 - 59)};
     }
 }
 

@@ -2,10 +2,20 @@
 //
 // A block is `lanes` sites x `units` threads, thread t = lane*units + unit;
 // a unit is one RHS (FP64) or one RHS pair (FP32 paired layout, LANES = 2).
-// Each thread passes per-RHS partial sums (FP64); the block sums them over
-// its lanes in a fixed tree, writes one partial per RHS to global scratch,
-// and the last block to finish (atomic ticket) sums the block partials in a
-// fixed order.  The result for an RHS never depends on the other RHS.
+// Each thread passes per-RHS partial sums; the block sums them over its
+// lanes in a fixed tree, writes one partial per RHS to global scratch, and
+// the last block to finish (atomic ticket) sums the block partials in a fixed
+// order.  The result for an RHS never depends on the other RHS.
+//
+// The sums across threads run on 64-bit integers with an exponent (Sum): an
+// FP64 add holds GB300's FP64 pipe for 64 cycles a warp, so the trees of a
+// 384-thread block with 8 values a thread, the last block's pass over 300
+// partials and the FP64 conversions around them took most of a reduction
+// kernel on a small lattice (16x8^3, 12 RHS: the three of a BiCGStab iteration
+// 20, 17 and 16 us, now 16, 13 and 10).  An integer add with alignment is
+// about 10 instructions.  Terms are aligned to the largest
+// one with its leading bit at 2^kLead or above, so a sum of N terms is off by
+// at most N 2^-kLead of its largest term (FP64 adds: N 2^-53 of the sum).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -79,6 +89,59 @@ __device__ __forceinline__ double2 zmul(double2 a, double2 b)
 }
 __device__ __forceinline__ bool zfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
+// ---- sums of floats or doubles on integers ------------------------------------
+
+// m 2^e; e = kSumBad: an infinity or NaN went in
+struct Sum {
+    long long m;
+    int e;
+};
+constexpr int kSumZero = -(1 << 20), kSumBad = 1 << 20;
+
+// x with its leading bit at 2^lead
+__device__ __forceinline__ Sum sum_of(float x, int lead)
+{
+    const int b = __float_as_int(x), be = (b >> 23) & 0xff;
+    const int f = b & 0x7fffff;
+    const long long m = (long long)(be ? f | 0x800000 : f) << (lead - 23);
+    const int e = (be ? be : 1) - 127 - lead;
+    return {b < 0 ? -m : m, be == 0xff ? kSumBad : m ? e : kSumZero};
+}
+__device__ __forceinline__ Sum sum_of(double x, int lead)
+{
+    const long long b = __double_as_longlong(x);
+    const int be = (int)(b >> 52) & 0x7ff;
+    long long m = b & 0xfffffffffffffll;
+    if (be) m |= 1ll << 52;
+    const int e = (be ? be : 1) - 1023 - lead;
+    m = lead >= 52 ? m << (lead - 52) : m >> (52 - lead);
+    return {b < 0 ? -m : m, be == 0x7ff ? kSumBad : m ? e : kSumZero};
+}
+__device__ __forceinline__ Sum add(Sum a, Sum b)
+{
+    const int e = max(a.e, b.e);
+    return {(a.m >> min(e - a.e, 63)) + (b.m >> min(e - b.e, 63)), e};
+}
+// leading bit brought down to 2^lead or below (no bit is lost upwards)
+__device__ __forceinline__ Sum cap(Sum a, int lead)
+{
+    const int top = 63 - __clzll(a.m < 0 ? ~a.m : a.m);
+    const int n = top > lead ? top - lead : 0;
+    return {a.m >> n, a.e >= kSumBad ? a.e : a.e + n};
+}
+__device__ __forceinline__ double value(Sum a)
+{
+    if (a.e >= kSumBad) return __longlong_as_double(0x7ff8000000000000ll);
+    if (!a.m) return 0.0;
+    const double d = (double)a.m;
+    const int x = ((__double2hiint(d) >> 20) & 0x7ff) + a.e;
+    if (x < 1 || x > 2046) return scalbn(d, a.e);  // subnormal or infinite
+    return __hiloint2double(__double2hiint(d) + a.e * (1 << 20), __double2loint(d));
+}
+
+// bit for the leading term that leaves room for n additions in 63 bits
+__device__ __forceinline__ int lead_for(int n) { return 61 - (32 - __clz(n - 1 > 0 ? n - 1 : 1)); }
+
 // ---- per-RHS BiCGStab scalar recurrences, applied by the last block ----------
 
 // alpha = rho / <rhat, v>
@@ -94,6 +157,7 @@ __device__ __forceinline__ void finish_alpha(RhsState &S, double re, double im)
         S.active = 0;
     } else {
         S.alpha = zdiv(S.rho, rv);
+        S.alpha_f = make_float2((float)S.alpha.x, (float)S.alpha.y);
     }
 }
 
@@ -135,15 +199,18 @@ __device__ __forceinline__ void finish_omega_shadow(RhsState &S, double ts_re, d
         return;
     }
     S.omega = tt > 0 ? make_double2(ts_re / tt, ts_im / tt) : make_double2(0.0, 0.0);
+    S.omega_f = make_float2((float)S.omega.x, (float)S.omega.y);
     const double2 wrt = zmul(S.omega, S.rt);
     const double2 rho_new = make_double2(S.rs.x - wrt.x, S.rs.y - wrt.y);
     if ((S.omega.x == 0.0 && S.omega.y == 0.0) || (rho_new.x == 0.0 && rho_new.y == 0.0)) {
         S.brk = 1;
         S.beta = make_double2(0.0, 0.0);
     } else {
-        S.beta = zmul(zdiv(rho_new, S.rho), zdiv(S.alpha, S.omega));
+        // one division (each is some 20 FP64 instructions of 64 cycles)
+        S.beta = zdiv(zmul(rho_new, S.alpha), zmul(S.rho, S.omega));
         S.rho = rho_new;
     }
+    S.beta_f = make_float2((float)S.beta.x, (float)S.beta.y);
 }
 
 // iteration count, convergence, cap, breakdown; beta = (rho'/rho)(alpha/omega)
@@ -205,6 +272,8 @@ __device__ __forceinline__ void finish_init(RhsState &S, double bb)
     S.alpha = make_double2(1.0, 0.0);
     S.omega = make_double2(1.0, 0.0);
     S.beta = make_double2(0.0, 0.0);
+    S.alpha_f = S.omega_f = make_float2(1.f, 0.f);
+    S.beta_f = make_float2(0.f, 0.f);
     S.iters = 0;
     S.brk = 0;
     if (!isfinite(bb)) {
@@ -230,6 +299,7 @@ __device__ __forceinline__ void finish_cg_gamma(RhsState &S, double zz, int firs
         S.active = 0;
     } else {
         S.beta = make_double2(first ? 0.0 : zz / S.rho.x, 0.0);
+        S.beta_f = make_float2((float)S.beta.x, 0.f);
         S.rho = make_double2(zz, 0.0);
     }
 }
@@ -246,6 +316,7 @@ __device__ __forceinline__ void finish_cg_alpha(RhsState &S, double ww)
         S.active = 0;
     } else {
         S.alpha = make_double2(S.rho.x / ww, 0.0);
+        S.alpha_f = make_float2((float)S.alpha.x, 0.f);
     }
 }
 
@@ -267,54 +338,69 @@ __device__ __forceinline__ void finish_cg_update(RhsState &S, double rr, int max
     }
 }
 
-// Block + grid reduction of NV doubles per RHS for LANES RHS per thread
-// (v[L*NV + k] belongs to RHS LANES*unit + L).  Returns true in exactly one
-// thread per unit (lane 0 of the last block), with the totals in v.  The
-// block tree runs kRedChunk values at a time through shared memory; each
-// value's summation order is the same fixed tree whatever NV is.
-constexpr int kRedChunk = 4;
+// Block + grid reduction of NV values per RHS for LANES RHS per thread
+// (v[L*NV + k] belongs to RHS LANES*unit + L; floats or doubles).  Returns
+// true in the threads of the last block; its thread r (r < the RHS count) then
+// has the totals of RHS r in `tot`, so the scalar recurrences of all RHS run
+// side by side in one or two warps.
 
+// sum over the lanes of a block: one barrier a level, the levels taking turns
+// between two regions of `sh`; the result is in the threads of lane 0
 template <int W>
-__device__ __forceinline__ void block_tree(double v[W], double *sh, const Cfg c, int t, int units,
+__device__ __forceinline__ void block_tree(Sum (&v)[W], long long *shm, int *she, const Cfg c, int t, int units,
                                            int lane)
 {
+    constexpr int kHalf = kMaxBlock / 2;
+    int region = 0;
+    for (int w = c.lanes / 2; w > 0; w >>= 1, region ^= 1) {
+        const int base = region ? kHalf * W : 0;
+        if (lane >= w && lane < 2 * w)
 #pragma unroll
-    for (int k0 = 0; k0 < W; k0 += kRedChunk) {
-#pragma unroll
-        for (int k = 0; k < kRedChunk; k++)
-            if (k0 + k < W) sh[t * kRedChunk + k] = v[k0 + k];
+            for (int k = 0; k < W; k++) {
+                shm[base + (t - w * units) + k * w * units] = v[k].m;
+                she[base + (t - w * units) + k * w * units] = v[k].e;
+            }
         __syncthreads();
-        for (int w = c.lanes / 2; w > 0; w >>= 1) {
-            if (lane < w)
+        if (lane < w)
 #pragma unroll
-                for (int k = 0; k < kRedChunk; k++)
-                    if (k0 + k < W) sh[t * kRedChunk + k] += sh[(t + w * units) * kRedChunk + k];
-            __syncthreads();
-        }
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < kRedChunk; k++)
-                if (k0 + k < W) v[k0 + k] = sh[t * kRedChunk + k];
-        __syncthreads();
+            for (int k = 0; k < W; k++)
+                v[k] = add(v[k], Sum{shm[base + t + k * w * units], she[base + t + k * w * units]});
     }
 }
 
-template <int NV, int LANES>
-__device__ bool reduce_last(double v[LANES * NV], const Cfg c, double *partials,
-                            unsigned int *counter, int units)
+struct __align__(16) Partial {
+    long long m;
+    int e, pad;
+};
+static_assert(sizeof(Partial) == 16, "two doubles of the scratch each");
+
+template <int NV, int LANES, typename T>
+__device__ __forceinline__ bool reduce_last(const T (&in)[LANES * NV], const Cfg c, double *partials,
+                                            unsigned int *counter, int units, double (&tot)[NV])
 {
-    static_assert(NV <= kRedWidth, "per-RHS partials hold kRedWidth values");
+    static_assert(2 * NV <= kRedWidth, "per-RHS partials hold kRedWidth doubles");
     constexpr int W = LANES * NV;
-    __shared__ double sh[kMaxBlock * kRedChunk];
+    __shared__ long long shm[(kMaxBlock / 2 + kMaxBlock / 4) * W];
+    __shared__ int she[(kMaxBlock / 2 + kMaxBlock / 4) * W];
     __shared__ bool last;
     const int t = threadIdx.x, u = t % units, lane = t / units;
-    block_tree<W>(v, sh, c, t, units, lane);
-    if (lane == 0)
+    Partial *part = reinterpret_cast<Partial *>(partials);
+    constexpr int kStride = kMaxRhs * kRedWidth / 2;  // per block
+    const int lead2 = lead_for((int)gridDim.x);
+    {
+        const int lead1 = lead_for(c.lanes);
+        Sum v[W];
 #pragma unroll
-        for (int L = 0; L < LANES; L++)
+        for (int k = 0; k < W; k++) v[k] = sum_of(in[k], lead1);
+        block_tree<W>(v, shm, she, c, t, units, lane);
+        if (lane == 0)
 #pragma unroll
-            for (int k = 0; k < NV; k++)
-                partials[((long long)blockIdx.x * kMaxRhs + LANES * u + L) * kRedWidth + k] = v[L * NV + k];
+            for (int k = 0; k < W; k++) {
+                const Sum s = cap(v[k], lead2);
+                part[(long long)blockIdx.x * kStride + (LANES * u + k / NV) * (kRedWidth / 2) + k % NV] =
+                    Partial{s.m, s.e, 0};
+            }
+    }
     __threadfence();
     __syncthreads();
     if (t == 0) last = (atomicAdd(counter, 1u) == (unsigned)(gridDim.x - 1));
@@ -322,21 +408,39 @@ __device__ bool reduce_last(double v[LANES * NV], const Cfg c, double *partials,
     if (!last) return false;
     __threadfence();
     // last block: lane l sums blocks l, l+lanes, ... in order, then a fixed tree
-    double acc[W];
+    Sum acc[W];
 #pragma unroll
-    for (int k = 0; k < W; k++) acc[k] = 0;
+    for (int k = 0; k < W; k++) acc[k] = Sum{0, kSumZero};
+#pragma unroll 4
     for (int b = lane; b < (int)gridDim.x; b += c.lanes)
 #pragma unroll
-        for (int L = 0; L < LANES; L++)
-#pragma unroll
-            for (int k = 0; k < NV; k++)
-                acc[L * NV + k] += __ldcg(partials + ((long long)b * kMaxRhs + LANES * u + L) * kRedWidth + k);
-    block_tree<W>(acc, sh, c, t, units, lane);
+        for (int k = 0; k < W; k++) {
+            const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(
+                part + (long long)b * kStride + (LANES * u + k / NV) * (kRedWidth / 2) + k % NV));
+            acc[k] = add(acc[k], Sum{w.x, (int)w.y});
+        }
+    block_tree<W>(acc, shm, she, c, t, units, lane);
     if (t == 0) *counter = 0u;
-    if (lane != 0) return false;
+    __syncthreads();
+    if (lane == 0)
 #pragma unroll
-    for (int k = 0; k < W; k++) v[k] = acc[k];
+        for (int k = 0; k < W; k++) {
+            shm[(LANES * u + k / NV) * NV + k % NV] = acc[k].m;
+            she[(LANES * u + k / NV) * NV + k % NV] = acc[k].e;
+        }
+    __syncthreads();
+    if (t < LANES * units)
+#pragma unroll
+        for (int k = 0; k < NV; k++) tot[k] = value(Sum{shm[t * NV + k], she[t * NV + k]});
     return true;
+}
+
+// in the last block, after thread r has finished RHS r: how many still iterate
+__device__ __forceinline__ void count_active(const RhsState *st, int nrhs, int *n_active)
+{
+    const int t = threadIdx.x;
+    const int k = __syncthreads_count(t < nrhs && st[t].active != 0);
+    if (t == 0) *n_active = k;
 }
 
 }  // namespace dp

@@ -147,13 +147,15 @@ __global__ void __launch_bounds__(kMaxBlock)
             acc[0] += sr * R * R;
         }
     }
-    if (!reduce_last<1, 1>(acc, c, partials, counter, n)) return;
-    if (!refined(st[r])) return;
-    const double sc = sqrt(acc[0]);
-    st[r].scale = sc;
+    double tot[1];
+    if (!reduce_last<1, 1>(acc, c, partials, counter, n, tot)) return;
+    if ((int)threadIdx.x >= n || !refined(st[threadIdx.x])) return;
+    RhsState &S = st[threadIdx.x];
+    const double sc = sqrt(tot[0]);
+    S.scale = sc;
     if (!isfinite(sc)) {
-        st[r].status = 3;
-        st[r].active = 0;
+        S.status = 3;
+        S.active = 0;
     }
 }
 

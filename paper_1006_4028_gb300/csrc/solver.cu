@@ -571,7 +571,7 @@ dp_status Batch::admit(Job *j)
     }
     CK(cudaMemcpyAsync(outer + s0, &hs[s0], sizeof(RhsState) * j->ncomp, cudaMemcpyHostToDevice, st_));
     CK(blas_residual64(bc_, bh, y64, r64, Vh, n, outer, mask_d, st_));
-    c->launches += 5;
+    c->launches += 4;
     CK(cudaStreamSynchronize(st_));
     return DP_OK;
 }
@@ -591,12 +591,11 @@ dp_status Batch::bicgstab(int max_iter, int *iters_done)
         dp_status s = apply_mhat_dag(c, opin, opin_adj, sp, in.rh, in.rh2, in.s, in.to, inner);
         if (s != DP_OK) return s;
         CK(blas32_alpha(bc, in.rh2, in.p, Vh, n, inner, st_));
-        CK(blas_count_active(bc, inner, n, st_));
         c->launches += 1;
     } else {
         CK(blas_bicg_init(bc, pr, in.rh, in.r, in.rh, in.p, in.v, in.x, Vh, n, inner, 0.0, st_));
     }
-    c->launches += 2;
+    c->launches += 1;
     CK(cudaMemcpyAsync(hnact_, bc.n_active, sizeof(int), cudaMemcpyDeviceToHost, st_));
     CK(cudaStreamSynchronize(st_));
     int it = 0;
@@ -622,7 +621,7 @@ dp_status Batch::bicgstab(int max_iter, int *iters_done)
             CK(blas32_update_pa(bc, in.x, in.r, in.p, in.s, in.t, in.v, in.rh2, Vh, n, inner,
                                 max_iter, st_));
         }
-        c->launches += 4;
+        c->launches += 3;
         return DP_OK;
     };
     auto body = [&](int first) -> dp_status {
@@ -652,7 +651,7 @@ dp_status Batch::bicgstab(int max_iter, int *iters_done)
             CK(blas_bicg_update(bc, pr, in.x, in.r, in.p, in.s, in.t, in.rh, Vh, n, inner, max_iter,
                                 st_));
         }
-        c->launches += 6;
+        c->launches += 5;
         return DP_OK;
     };
     const bool graphs = opts.use_graph && !c->timing;
@@ -675,7 +674,7 @@ dp_status Batch::bicgstab(int max_iter, int *iters_done)
                 graph_max_iter = max_iter;
             }
             CK(cudaGraphLaunch(graph, st_));
-            c->launches += fused ? 8 : opin.xw ? 12 : 10;
+            c->launches += fused ? 7 : opin.xw ? 11 : 9;
         }
         it++;
         if (it >= max_iter) break;
@@ -740,7 +739,7 @@ dp_status Batch::sap_gcr(int max_iter, int *iters_done)
     BlasCtx &bc = bc_;
     const long long Vh = f->g.Vh;
     CK(blas_bicg_init(bc, 1, in.rh, in.r, in.rh, in.p, in.v, in.x, Vh, n, inner, 0.0, st_));
-    c->launches += 2;
+    c->launches += 1;
     CK(cudaMemcpyAsync(hnact_, bc.n_active, sizeof(int), cudaMemcpyDeviceToHost, st_));
     CK(cudaStreamSynchronize(st_));
     *iters_done = 0;
@@ -760,7 +759,7 @@ dp_status Batch::sap_gcr(int max_iter, int *iters_done)
             CK(blas32_normalise(bc, wk[k], zk[k], Vh, n, inner, nrm2_d, st_));
             CK(blas32_dotv(bc, wk[k], in.r, Vh, n, inner, coef_d, st_));
             CK(blas32_gcr_update(bc, in.x, in.r, zk[k], wk[k], Vh, n, inner, coef_d, max_iter, st_));
-            c->launches += 2 * k + 5;
+            c->launches += 2 * k + 4;
             it++;
             CK(cudaMemcpyAsync(hnact_, bc.n_active, sizeof(int), cudaMemcpyDeviceToHost, st_));
             CK(cudaStreamSynchronize(st_));
@@ -832,7 +831,7 @@ dp_status Batch::cgne(int max_iter, int *iters_done)
     const int pr = opin.pr;
     const long long Vh = f->g.Vh;
     CK(blas_bicg_init(bc, pr, in.rh, in.r, in.rh, in.p, in.v, in.x, Vh, n, inner, 0.0, st_));
-    c->launches += 2;
+    c->launches += 1;
     CK(cudaMemcpyAsync(hnact_, bc.n_active, sizeof(int), cudaMemcpyDeviceToHost, st_));
     CK(cudaStreamSynchronize(st_));
     int it = 0;
@@ -850,7 +849,7 @@ dp_status Batch::cgne(int max_iter, int *iters_done)
         if (s != DP_OK) return s;
         CK(blas_cg_alpha(bc, pr, in.v, Vh, n, inner, st_));
         CK(blas_cg_update(bc, pr, in.x, in.r, in.p, in.v, Vh, n, inner, max_iter, st_));
-        c->launches += 5;
+        c->launches += 4;
         return DP_OK;
     };
     const bool graphs = opts.use_graph && !c->timing;
@@ -873,7 +872,7 @@ dp_status Batch::cgne(int max_iter, int *iters_done)
                 graph_max_iter = max_iter;
             }
             CK(cudaGraphLaunch(graph, st_));
-            c->launches += opin.xw ? 12 : 10;
+            c->launches += opin.xw ? 11 : 9;
         }
         it++;
         if (it >= max_iter) break;
@@ -987,7 +986,7 @@ dp_status Batch::round()
         Timed tm(c, st_, "outer_blas");
         CK(blas_residual64(bc_, bh, y64, r64, Vh, n, outer, nullptr, st_));
     }
-    c->launches += 3;
+    c->launches += 2;
     return DP_OK;
 }
 

@@ -190,14 +190,14 @@ cudaError_t launch_point_source(const Geom &g, const SlotInfo *slots_dev, int nr
 // doubles with P = contract_blocks_per_slice(g); prop_lex: NULL or
 // [nrhs][V][12] complex128 of the restored propagator
 int contract_blocks_per_slice(const Geom &g);
-// only RHS with mask[r] != 0 contribute (mask NULL: all)
+// only RHS r0 .. r0 + nr (nr = 0: all) with mask[r] != 0 contribute (mask NULL: all)
 // cap_dev (optional): C_AP(y0) = sum tr[gamma_0 S S^dag] per group, same
 // layout as cpp_dev; partials then needs 2 * T * P * n_mass doubles
 cudaError_t launch_restore_contract(const double2 *xe, const double2 *xo, const Geom &g, int nrhs,
                                     const double *alpha, const SlotInfo *slots_dev, int ngroups,
                                     const int *t_src_dev, const int *mask, double *cpp_dev,
                                     double *partials, double2 *prop_lex, cudaStream_t st,
-                                    double *cap_dev = nullptr);
+                                    double *cap_dev = nullptr, int r0 = 0, int nr = 0);
 // heavy-light C(y0) = -sum_{y vec} tr[S_h S_l^dag] of two groups' propagators
 // (slots slot_h.. and slot_l.., 12 each, groups gh, gl for their profiles);
 // out_dev [T][2] (re, im), y0 relative to t_src; partials: 2 * T * P doubles

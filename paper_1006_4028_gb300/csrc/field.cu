@@ -11,6 +11,7 @@
 //    source, reduced per time slice in a fixed order (deterministic).
 #include "cplx.cuh"
 #include "dp_internal.h"
+#include "slice_sum.cuh"
 
 namespace dp {
 namespace {
@@ -192,91 +193,81 @@ __global__ void k_point_source(Geom g, const SlotInfo *slots, int n, const int *
 
 constexpr int kContractBlock = 256;
 
-// grid (P, T): block (p, t) sums |S'|^2/alpha_B^2 over its share of slice t,
-// per group; partials[(t*P + p)*ng + grp].  With `ap`, also the gamma_0
-// bilinear tr[gamma_0 S S^dag] (chiral basis: gamma_0 = -1 between spins 0,2
-// and 1,3, i.e. -2 Re sum_c [S(0,c) S(2,c)* + S(1,c) S(3,c)*] per RHS) into
-// partials[T*P*ng + (t*P + p)*ng + grp]
-__global__ void __launch_bounds__(kContractBlock)
+// grid (P, T): block (p, t) sums |S'|^2/alpha_B^2 over its share of slice t for
+// the RHS r0 .. r0 + nr, per group; partials[(t*P + p)*ng + grp] (see
+// slice_sum.cuh).  OUT: restore each component (S = S'/alpha_B) instead, into
+// `prop` if given and with `ap` also the gamma_0 bilinear tr[gamma_0 S S^dag]
+// (chiral basis: gamma_0 = -1 between spins 0,2 and 1,3, i.e. -2 Re sum_c
+// [S(0,c) S(2,c)* + S(1,c) S(3,c)*] per RHS) into
+// partials[T*P*ng + (t*P + p)*ng + grp]; the same arithmetic serves spinors
+// and profiles beyond the integer sums' range.
+//
+// 32x16^3, 36 RHS, 0.906 GB: 0.200 ms = 4.5 TB/s (0.134 at the copy rate; 1.166 with 64 blocks
+// and 48 FP64 operations and a division a spinor); 48x24^3, 12 RHS: 0.33 ms (1.10).
+template <bool OUT>
+__global__ void __launch_bounds__(kSliceThreads)
     k_contract(const double2 *xe, const double2 *xo, Geom g, int n, const double *alpha,
-               const SlotInfo *slots, const int *mask, int ng, double *partials, double2 *prop,
+               const SlotInfo *slots, const int *mask, int r0, int nr, int ng, double *partials, double2 *prop,
                int ap)
 {
+    extern __shared__ double iw[];
+    __shared__ int grp[kMaxRhs];
     const int P = gridDim.x, p = blockIdx.x, t = blockIdx.y;
-    const long long Vs = g.Vh / g.T;  // half-sites per slice per parity
-    const long long chunk = (Vs + P - 1) / P;
-    const long long j0 = p * chunk, j1 = min(Vs, j0 + chunk);
-    const int nm = ng;
-    const long long cs = g.Vh * n;
-    double loc[kMaxGroups], lap[kMaxGroups];
-    for (int m = 0; m < kMaxGroups; m++) loc[m] = lap[m] = 0;
-    const long long work = (j1 > j0 ? j1 - j0 : 0) * n;
-    for (long long e = threadIdx.x; e < work; e += blockDim.x) {
-        const long long s = (long long)t * Vs + j0 + e / n;
-        const int r = (int)(e % n);
-        if (mask && !mask[r]) continue;
-        const int xh = (int)(s % g.Lxh);
-        long long q = s / g.Lxh;
-        const int y = (int)(q % g.Ly);
-        q /= g.Ly;
-        const int z = (int)(q % g.Lz);
-        const int grp = slots[r].group;
-        const double *al = alpha + (long long)grp * 4 * g.Lmax;
-        const double base = al[0 * g.Lmax + t] * al[2 * g.Lmax + y] * al[3 * g.Lmax + z];
-        double acc = 0, acc_ap = 0;
+    const SliceShare h = slice_share(g, r0, nr);
+    for (int k = threadIdx.x; k < nr; k += blockDim.x)
+        grp[r0 + k] = mask && !mask[r0 + k] ? -1 : slots[r0 + k].group;
+    if (!OUT) slice_weights(iw, g, alpha, ng);
+    __syncthreads();
+    const long long Vs = g.Vh / g.T, cs = g.Vh * n;
+    const int m = h.on ? grp[h.r] : -1;
+    const double *al = alpha + (long long)(m < 0 ? 0 : m) * 4 * g.Lmax;
+    double sum[2] = {0, 0};  // OUT: the bilinear, else the weighted sum without 1/alpha_t^2; general arithmetic
+    for (int j = h.j0 + h.lane; m >= 0 && j < h.j1; j += h.lanes) {
+        const int xh = j % g.Lxh, q = j / g.Lxh, y = q % g.Ly, z = q / g.Ly;
+        const long long s = t * Vs + j;
+        double2 c[2][12];
+#pragma unroll
+        for (int par = 0; par < 2; par++)
+#pragma unroll
+            for (int k = 0; k < 12; k++) c[par][k] = __ldg((par ? xo : xe) + k * cs + s * n + h.r);
+#pragma unroll
         for (int par = 0; par < 2; par++) {
             const int x = 2 * xh + ((t + y + z + par) & 1);
-            const double inv = 1.0 / (base * al[1 * g.Lmax + x]);
-            const double2 *v = (par ? xo : xe) + s * n + r;
-            double2 *pd = prop ? prop + ((long long)r * g.V + 2 * s + (x & 1)) * 12 : nullptr;
-            double sp = 0;
-            double2 c[12];
-            for (int k = 0; k < 12; k++) {
-                c[k] = v[k * cs];
-                c[k].x *= inv;
-                c[k].y *= inv;
-                sp = fmx(c[k].x, c[k].x, sp);
-                sp = fmx(c[k].y, c[k].y, sp);
-                if (pd) pd[k] = c[k];
-            }
-            acc += sp;
-            if (ap) {
-                double b = 0;  // Re sum_c [S(0,c) S(2,c)* + S(1,c) S(3,c)*]
-                for (int k = 0; k < 6; k++) {
-                    b = fmx(c[k].x, c[k + 6].x, b);
-                    b = fmx(c[k].y, c[k + 6].y, b);
+            if (!OUT) {
+                const double *w3 = iw + m * 3 * g.Lmax;
+                const double w = w3[g.Lmax + y] * w3[2 * g.Lmax + z] * w3[x];
+                double s2;
+                if (weight_ok(w) && norm2_int(c[par], s2)) {
+                    sum[0] = fmx(s2, w, sum[0]);
+                    continue;
                 }
-                acc_ap -= 2.0 * b;
             }
-        }
+            const double inv = 1.0 / (al[t] * al[2 * g.Lmax + y] * al[3 * g.Lmax + z] * al[g.Lmax + x]);
+            double2 *pd = OUT && prop ? prop + ((long long)h.r * g.V + 2 * s + (x & 1)) * 12 : nullptr;
+            double sp = 0, b = 0;  // b = Re sum_c [S(0,c) S(2,c)* + S(1,c) S(3,c)*]
 #pragma unroll
-        for (int m = 0; m < kMaxGroups; m++)
-            if (m == grp) {
-                loc[m] += acc;
-                lap[m] += acc_ap;
+            for (int k = 0; k < 12; k++) {
+                double2 &v = c[par][k];
+                v.x *= inv;
+                v.y *= inv;
+                sp = fmx(v.x, v.x, sp);
+                sp = fmx(v.y, v.y, sp);
+                if (pd) pd[k] = v;
+                if (OUT && ap && k >= 6) {
+                    b = fmx(c[par][k - 6].x, v.x, b);
+                    b = fmx(c[par][k - 6].y, v.y, b);
+                }
             }
-    }
-    __shared__ double sh[kContractBlock];
-    for (int m = 0; m < nm; m++) {
-        sh[threadIdx.x] = loc[m];
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
+            sum[1] += sp;
+            if (OUT) sum[0] -= 2.0 * b;
         }
-        if (threadIdx.x == 0) partials[((long long)t * P + p) * nm + m] = sh[0];
-        __syncthreads();
-        if (!ap) continue;
-        sh[threadIdx.x] = lap[m];
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0)
-            partials[(long long)g.T * P * nm + ((long long)t * P + p) * nm + m] = sh[0];
-        __syncthreads();
     }
+    double tot[2];
+    slice_totals<2>(sum, h.lanes, nr, r0, grp, ng, tot);
+    if ((int)threadIdx.x >= ng) return;
+    const double at = alpha[(long long)threadIdx.x * 4 * g.Lmax + t];
+    partials[((long long)t * P + p) * ng + threadIdx.x] = OUT ? tot[1] : tot[1] + over_square(tot[0], at);
+    if (OUT && ap) partials[(long long)g.T * P * ng + ((long long)t * P + p) * ng + threadIdx.x] = tot[0];
 }
 
 // cpp[m][(t - t_src[m]) mod T] = -sum_p partials[t][p][m], summed in p order;
@@ -446,28 +437,48 @@ cudaError_t launch_contract_hl(const double2 *xe, const double2 *xo, const Geom 
     return cudaGetLastError();
 }
 
-// partials must hold T * P * n_mass doubles, P = contract_blocks_per_slice(g)
+// Blocks per slice: four blocks an SM over all slices where that leaves each
+// at least 32 half-sites, and at most 1024 half-sites a block.  (One block per 1024
+// half-sites left a 32x16^3 lattice with 64 blocks for 152 SMs.)
 int contract_blocks_per_slice(const Geom &g)
 {
     const long long Vs = g.Vh / g.T;
-    long long P = (Vs + 1023) / 1024;
+    const long long fill = (4 * 152 + g.T - 1) / g.T, most = (Vs + 31) / 32;
+    long long P = std::max((Vs + 1023) / 1024, std::min(fill, most));
     if (P < 1) P = 1;
     if (P > 64) P = 64;
     return (int)P;
 }
 
+namespace {
+// the contraction's first pass; partials: T * P * ngroups doubles (twice that with ap)
+cudaError_t contract_pass(const double2 *xe, const double2 *xo, const Geom &g, int n, const double *alpha,
+                          const SlotInfo *slots, const int *mask, int r0, int nr, int ng, double *partials,
+                          double2 *prop, int ap, cudaStream_t st)
+{
+    const int P = contract_blocks_per_slice(g), threads = slice_lanes(nr) * nr;
+    const size_t smem = slice_smem(g, ng);
+    const dim3 grid(P, g.T);
+    // (the inverse squares of many groups on very long extents: general arithmetic)
+    if (prop || ap || smem > 32 * 1024)
+        k_contract<true><<<grid, threads, 0, st>>>(xe, xo, g, n, alpha, slots, mask, r0, nr, ng, partials, prop, ap);
+    else
+        k_contract<false><<<grid, threads, smem, st>>>(xe, xo, g, n, alpha, slots, mask, r0, nr, ng, partials,
+                                                       nullptr, 0);
+    return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_restore_contract(const double2 *xe, const double2 *xo, const Geom &g, int nrhs,
                                     const double *alpha, const SlotInfo *slots_dev, int ngroups,
                                     const int *t_src_dev, const int *mask, double *cpp_dev,
                                     double *partials, double2 *prop_lex, cudaStream_t st,
-                                    double *cap_dev)
+                                    double *cap_dev, int r0, int nr)
 {
     if (ngroups < 1 || ngroups > kMaxGroups) return cudaErrorInvalidValue;
     const int P = contract_blocks_per_slice(g);
-    dim3 grid(P, g.T);
-    k_contract<<<grid, kContractBlock, 0, st>>>(xe, xo, g, nrhs, alpha, slots_dev, mask, ngroups,
-                                                partials, prop_lex, cap_dev ? 1 : 0);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = contract_pass(xe, xo, g, nrhs, alpha, slots_dev, mask, r0, nr > 0 ? nr : nrhs, ngroups, partials,
+                                  prop_lex, cap_dev ? 1 : 0, st);
     if (e != cudaSuccess) return e;
     const int tot = g.T * ngroups;
     k_contract_final<<<(tot + 127) / 128, 128, 0, st>>>(partials, P, g.T, ngroups, t_src_dev, cpp_dev,
@@ -635,11 +646,8 @@ extern "C" dp_status dp_restore_contract_noalloc(dp_ctx *ctx, dp_field field, in
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(tsrc_d, tsrc, sizeof(int) * n_groups, cudaMemcpyHostToDevice, c.stream);
     if (e == cudaSuccess) {
-        dim3 grid(P, g.T);
-        k_contract<<<grid, kContractBlock, 0, c.stream>>>((const double2 *)xe, (const double2 *)xo, g, n,
-                                                          alpha_d, slots_d, nullptr, n_groups, part_d,
-                                                          nullptr, 0);
-        e = cudaGetLastError();
+        e = contract_pass((const double2 *)xe, (const double2 *)xo, g, n, alpha_d, slots_d, nullptr, 0, n, n_groups,
+                          part_d, nullptr, 0, c.stream);
     }
     if (e == cudaSuccess) {
         const int tot = g.T * n_groups;

@@ -1231,7 +1231,7 @@ dp_status Batch::harvest(std::vector<Job *> &finished)
         }
         CK(launch_restore_contract(sp == 0 ? x : y64, sp == 0 ? y64 : x, g, n, alpha_d, slots_d,
                                    kMaxGroups, tsrc_d, mask_d, cpp_d, cpart, prop_d, st_,
-                                   j->cap_dst ? cap_d : nullptr));
+                                   j->cap_dst ? cap_d : nullptr, j->slot0, j->ncomp));
         if (j->cpp_dst) CK(launch_cpp_commit(cpp_d + (size_t)tab * g.T, j->cpp_dst, g.T, j->accumulate, st_));
         if (j->cap_dst) CK(launch_cpp_commit(cap_d + (size_t)tab * g.T, j->cap_dst, g.T, j->accumulate, st_));
         if (j->cpp_host) CK(cudaMemcpyAsync(j->cpp_host, cpp_d + (size_t)tab * g.T, sizeof(double) * g.T, cudaMemcpyDeviceToHost, st_));

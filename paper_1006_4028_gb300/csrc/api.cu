@@ -118,10 +118,21 @@ Shape Ctx::launch_shape(long long Vh, int prec, int link_fmt, int nrhs)
     std::lock_guard<std::mutex> lk(mu);
     auto it = tuned.find(TuneKey{Vh, prec, link_fmt, nrhs});
     if (it != tuned.end()) return it->second;
+    // FP32, one RHS pair per thread: the spinor-staged kernel with 64 threads is
+    // the fastest or level with it at every size (times of A^-1 D in us, direct
+    // with 64 threads against it: 12 RHS on 16x8^3 10.1/8.3, 20x12x10x14
+    // 18.6/18.6, 24x16x12^2 34.6/28.7, 32x16^3 82/57, 48x24^3 381/254; 48 RHS on
+    // 32x16^3 291/194; 2 RHS there 16.4/14.8; 18-real links alike), but for
+    // 16-bit links on small lattices, whose unpacking the direct kernel hides
+    // better (16x8^3 8.9/10.4, 20x12x10x14 18.7/20.6, 24x16x12^2 32.5/28.9).
+    // Its thread index is 32 bits.
     Shape sh;
     sh.block = 64;
-    sh.rpt = prec == 0 ? 1 : 2;  // FP32: one RHS pair per thread
-    sh.stages = 0;
+    sh.rpt = prec == 0 ? 1 : 2;
+    const long long items = Vh * (nrhs / 2);
+    const bool h16 = link_fmt == LINK_H16_12 || link_fmt == LINK_B16_12;
+    if (prec != 0 && items < (1ll << 32) - 256 && (!h16 || items >= 128 * 1024)) sh.stages = 6;
+    sh.tuned = false;
     return sh;
 }
 
@@ -883,6 +894,9 @@ dp_status dp_dslash_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile 
     if (block_threads > 0) block = block_threads;
     if (rhs_per_thread != 0) rpt = want_rpt;
     if (stages >= 0) stg = stages;
+    // a block size or RHS count of the caller's that the default staging does
+    // not serve takes direct loads
+    else if (!sh.tuned && stg > 0 && !dslash_staged_ok(pr, lf, EPI_AINV, rpt, stg, block)) stg = 0;
     if (stg > 0 && !dslash_staged_ok(pr, lf, EPI_AINV, rpt, stg, block)) {
         c.release(hopd);
         set_error("dp_dslash_dev: shared-memory staging needs FP32 or 16-bit 12-real links, 2 RHS per "

@@ -133,6 +133,7 @@ struct Shape {
     int block = 64;
     int rpt = 1;
     int stages = 0;
+    bool tuned = true;  // from dp_autotune or dp_tune_set, not the default
 };
 
 // ---- clover (clover.cu) ----

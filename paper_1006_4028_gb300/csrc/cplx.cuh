@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "dp_internal.h"
 
 namespace dp {
@@ -227,6 +229,82 @@ __device__ __forceinline__ void load_link<LINK_B16_12, float>(const void *base, 
                                                              Cx<float> u[9])
 {
     load_link16<__nv_bfloat162>(base, Vh, site, mu, u);
+}
+
+// A link as stored (loaded ahead of its use, expanded by link_of): the 12-
+// and 18-real FP32 and the 16-bit formats
+template <int LF>
+struct RawLink {
+    float4 a[3];
+};
+template <>
+struct RawLink<LINK_F32_18> {
+    float4 a[4];
+    float2 b;
+};
+struct RawLink16 {
+    uint2 a[3];
+    float s;
+};
+template <>
+struct RawLink<LINK_H16_12> : RawLink16 {};
+template <>
+struct RawLink<LINK_B16_12> : RawLink16 {};
+
+template <int LF>
+__device__ __forceinline__ void load_raw(RawLink<LF> &w, const void *base, long long Vh, long long site, int mu)
+{
+    if constexpr (LF == LINK_F32_12) {
+        const float4 *l = static_cast<const float4 *>(base) + (long long)mu * 3 * Vh + site;
+#pragma unroll
+        for (int k = 0; k < 3; k++) w.a[k] = __ldg(l + k * Vh);
+    } else if constexpr (LF == LINK_F32_18) {
+        const float4 *l = static_cast<const float4 *>(base) + (long long)mu * 4 * Vh + site;
+#pragma unroll
+        for (int k = 0; k < 4; k++) w.a[k] = __ldg(l + k * Vh);
+        w.b = __ldg(reinterpret_cast<const float2 *>(static_cast<const float4 *>(base) + 16 * Vh) +
+                    (long long)mu * Vh + site);
+    } else {
+        const uint2 *l = static_cast<const uint2 *>(base) + (long long)mu * 3 * Vh + site;
+#pragma unroll
+        for (int k = 0; k < 3; k++) w.a[k] = __ldg(l + k * Vh);
+        w.s = __ldg(reinterpret_cast<const float *>(static_cast<const uint2 *>(base) + 12 * Vh) +
+                    (long long)mu * Vh + site);
+    }
+}
+
+template <int LF>
+__device__ __forceinline__ void link_of(const RawLink<LF> &w, Cx<float> u[9])
+{
+    if constexpr (LF == LINK_F32_18) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            u[2 * k] = {w.a[k].x, w.a[k].y};
+            u[2 * k + 1] = {w.a[k].z, w.a[k].w};
+        }
+        u[8] = {w.b.x, w.b.y};
+        return;
+    } else if constexpr (LF == LINK_F32_12) {
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            u[2 * k] = {w.a[k].x, w.a[k].y};
+            u[2 * k + 1] = {w.a[k].z, w.a[k].w};
+        }
+    } else {
+        using H2 = typename std::conditional<LF == LINK_H16_12, __half2, __nv_bfloat162>::type;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const float2 a = h2f<H2>(w.a[k].x), b = h2f<H2>(w.a[k].y);
+            u[2 * k] = {w.s * a.x, w.s * a.y};
+            u[2 * k + 1] = {w.s * b.x, w.s * b.y};
+        }
+    }
+    const Cx<float> a = cmul(u[1], u[5]) - cmul(u[2], u[4]);
+    const Cx<float> b = cmul(u[2], u[3]) - cmul(u[0], u[5]);
+    const Cx<float> c = cmul(u[0], u[4]) - cmul(u[1], u[3]);
+    u[6] = {a.re, -a.im};
+    u[7] = {b.re, -b.im};
+    u[8] = {c.re, -c.im};
 }
 
 // ---- clover blocks ------------------------------------------------------------

@@ -56,10 +56,10 @@ __device__ __forceinline__ int local_index(const SapParams &p, int lt, int lx, i
 // acc += hop from a neighbour held in shared memory (sm: [12][vbh] pairs)
 template <int LF, int MU, int SG>
 __device__ __forceinline__ void hop_local(C2 (&acc)[12], const ulonglong2 *sm, int vbh, int j,
-                                          const void *lk, long long Vh, long long lsite, float c)
+                                          const RawLink<LF> &w, float c)
 {
     Cx<float> u[9];
-    load_link<LF, float>(lk, Vh, lsite, MU, u);
+    link_of<LF>(w, u);
     const f2 C = bc(c), MC = bc(-c);
     C2 h[6];
 #pragma unroll
@@ -76,9 +76,13 @@ __device__ __forceinline__ void hop_local(C2 (&acc)[12], const ulonglong2 *sm, i
 }
 
 // sum of the hops of output site o (parity par) from the neighbours of the
-// other parity that lie inside the block; sm holds those neighbours
+// other parity that lie inside the block; sm holds those neighbours.  A hop
+// that leaves the block is computed with factor 0 from this thread's own slot
+// (its warp runs it for the other sites in any case), so there is no branch
+// and the link of the next hop is loaded before this one is computed: with
+// the hops under branches each waited for its link from L2.
 template <int LF>
-__device__ __forceinline__ void block_hops(const SapParams &p, const LocalSite &o, int par,
+__device__ __forceinline__ void block_hops(const SapParams &p, const LocalSite &o, int i, int par,
                                            const ulonglong2 *sm, int vbh, const float *ht,
                                            C2 (&acc)[12])
 {
@@ -87,34 +91,43 @@ __device__ __forceinline__ void block_hops(const SapParams &p, const LocalSite &
     const void *lown = p.links[par], *loth = p.links[1 - par];
 #pragma unroll
     for (int j = 0; j < 12; j++) acc[j] = {0ull, 0ull};
-    // neighbour global half index (no wrap inside a block)
-    auto gidx = [&](int t, int x, int y, int z) {
-        return ((((long long)t * g.Lz + z) * g.Ly + y) * g.Lx + x) >> 1;
+    const int st[4] = {g.Lz * g.Ly * g.Lx, 1, g.Lx, g.Ly * g.Lx};  // lexicographic strides
+    const int lc[4] = {o.lt, o.lx, o.ly, o.lz};
+    const int gc[4] = {o.t, o.x, o.y, o.z};
+    const long long lex = (((long long)o.t * g.Lz + o.z) * g.Ly + o.y) * g.Lx + o.x;
+    auto inside = [&](int mu, int back) { return back ? lc[mu] > 0 : lc[mu] + 1 < p.bs[mu]; };
+    auto fetch = [&](RawLink<LF> &w, int mu, int back) {
+        if (!back)
+            load_raw<LF>(w, lown, Vh, o.s, mu);
+        else  // (the link starts at the neighbour; outside the block: any of the other parity)
+            load_raw<LF>(w, loth, Vh, inside(mu, 1) ? (lex - st[mu]) >> 1 : o.s, mu);
     };
-    if (o.lt + 1 < p.bs[0])
-        hop_local<LF, 0, -1>(acc, sm, vbh, local_index(p, o.lt + 1, o.lx, o.ly, o.lz), lown, Vh, o.s,
-                             ht[0 * g.Lmax + o.t]);
-    if (o.lt > 0)
-        hop_local<LF, 0, +1>(acc, sm, vbh, local_index(p, o.lt - 1, o.lx, o.ly, o.lz), loth, Vh,
-                             gidx(o.t - 1, o.x, o.y, o.z), ht[1 * g.Lmax + o.t]);
-    if (o.lx + 1 < p.bs[1])
-        hop_local<LF, 1, -1>(acc, sm, vbh, local_index(p, o.lt, o.lx + 1, o.ly, o.lz), lown, Vh, o.s,
-                             ht[2 * g.Lmax + o.x]);
-    if (o.lx > 0)
-        hop_local<LF, 1, +1>(acc, sm, vbh, local_index(p, o.lt, o.lx - 1, o.ly, o.lz), loth, Vh,
-                             gidx(o.t, o.x - 1, o.y, o.z), ht[3 * g.Lmax + o.x]);
-    if (o.ly + 1 < p.bs[2])
-        hop_local<LF, 2, -1>(acc, sm, vbh, local_index(p, o.lt, o.lx, o.ly + 1, o.lz), lown, Vh, o.s,
-                             ht[4 * g.Lmax + o.y]);
-    if (o.ly > 0)
-        hop_local<LF, 2, +1>(acc, sm, vbh, local_index(p, o.lt, o.lx, o.ly - 1, o.lz), loth, Vh,
-                             gidx(o.t, o.x, o.y - 1, o.z), ht[5 * g.Lmax + o.y]);
-    if (o.lz + 1 < p.bs[3])
-        hop_local<LF, 3, -1>(acc, sm, vbh, local_index(p, o.lt, o.lx, o.ly, o.lz + 1), lown, Vh, o.s,
-                             ht[6 * g.Lmax + o.z]);
-    if (o.lz > 0)
-        hop_local<LF, 3, +1>(acc, sm, vbh, local_index(p, o.lt, o.lx, o.ly, o.lz - 1), loth, Vh,
-                             gidx(o.t, o.x, o.y, o.z - 1), ht[7 * g.Lmax + o.z]);
+    auto slot = [&](int mu, int back) {  // the neighbour's slot (no wrap inside a block)
+        const int d = back ? -1 : 1;
+        return inside(mu, back) ? local_index(p, o.lt + (mu == 0) * d, o.lx + (mu == 1) * d, o.ly + (mu == 2) * d,
+                                              o.lz + (mu == 3) * d)
+                                : i;
+    };
+    auto factor = [&](int mu, int back) {
+        return inside(mu, back) ? __ldg(ht + (2 * mu + back) * g.Lmax + gc[mu]) : 0.f;
+    };
+    RawLink<LF> w0, w1;
+    fetch(w0, 0, 0);
+    fetch(w1, 0, 1);
+    hop_local<LF, 0, -1>(acc, sm, vbh, slot(0, 0), w0, factor(0, 0));
+    fetch(w0, 1, 0);
+    hop_local<LF, 0, +1>(acc, sm, vbh, slot(0, 1), w1, factor(0, 1));
+    fetch(w1, 1, 1);
+    hop_local<LF, 1, -1>(acc, sm, vbh, slot(1, 0), w0, factor(1, 0));
+    fetch(w0, 2, 0);
+    hop_local<LF, 1, +1>(acc, sm, vbh, slot(1, 1), w1, factor(1, 1));
+    fetch(w1, 2, 1);
+    hop_local<LF, 2, -1>(acc, sm, vbh, slot(2, 0), w0, factor(2, 0));
+    fetch(w0, 3, 0);
+    hop_local<LF, 2, +1>(acc, sm, vbh, slot(2, 1), w1, factor(2, 1));
+    fetch(w1, 3, 1);
+    hop_local<LF, 3, -1>(acc, sm, vbh, slot(3, 0), w0, factor(3, 0));
+    hop_local<LF, 3, +1>(acc, sm, vbh, slot(3, 1), w1, factor(3, 1));
 }
 
 __device__ __forceinline__ void clover_inv_apply(const float4 *cl, long long Vh, long long s,
@@ -156,14 +169,19 @@ __device__ __forceinline__ void block_sum6(float (&v)[6], float *red)
 // and share its links and clover inverses in L1/L2), y = the blocks of this
 // colour (when the x-block count is even; otherwise all blocks, the other
 // colour exiting at once).  Shared memory per CTA: the block residual rho
-// (parity p), the correction delta (parity p) and t, then q (parity q / p).
+// (parity p) and t (parity q), which neighbours read; the correction delta and
+// q = Mhat_B rho stay in their thread's registers.  12 RHS on 32x16^3, 4 steps:
+// 0.312 ms (0.383 with delta and q in shared memory and branches round the hops;
+// the 80 KB of L1 that the smaller tile leaves matter: 0.368 with delta in
+// shared memory).  Bound: latency at 12 warps an SM; 128 registers for 16
+// warps spill (0.404).
 template <int LF>
 __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
 {
-    extern __shared__ ulonglong2 sm[];  // R, D: [12][vbh] (parity p); T: [12][vbh]
+    extern __shared__ ulonglong2 sm[];  // R: [12][vbh] (parity p); T: [12][vbh] (parity q)
     __shared__ float red[4 * 6];
     const int vbh = p.bs[0] * p.bs[1] * p.bs[2] * p.bs[3] / 2;
-    ulonglong2 *R = sm, *Tq = sm + 12 * vbh, *D = sm + 24 * vbh;
+    ulonglong2 *R = sm, *Tq = sm + 12 * vbh;
     // block coordinates and colour
     int b = blockIdx.y;
     int bx, by, bz, bt;
@@ -197,6 +215,9 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
     const int grp = p.grp_of[2 * q0];
     const float *ht = static_cast<const float *>(p.hop) + (long long)grp * 8 * p.g.Lmax;
     LocalSite sp_{}, sq_{};
+    C2 D[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) D[k] = {0ull, 0ull};
     if (live) {
         sp_ = local_site(p, i, pp, ot, ox, oy, oz);
         sq_ = local_site(p, i, qq, ot, ox, oy, oz);
@@ -204,7 +225,6 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
 #pragma unroll
         for (int k = 0; k < 12; k++) {
             R[k * vbh + i] = __ldg(src + k * cs);
-            D[k * vbh + i] = make_ulonglong2(0ull, 0ull);
         }
     }
     for (int it = 0; it < p.n_mr; it++) {
@@ -212,7 +232,7 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
         C2 acc[12];
         if (live) {
             // t (q-site i) = A_qq^-1 D_qp|_B rho
-            block_hops<LF>(p, sq_, qq, R, vbh, ht, acc);
+            block_hops<LF>(p, sq_, i, qq, R, vbh, ht, acc);
             clover_inv_apply(static_cast<const float4 *>(p.clov[qq][grp]), Vh, sq_.s, acc);
 #pragma unroll
             for (int k = 0; k < 12; k++) Tq[k * vbh + i] = make_ulonglong2(acc[k].re, acc[k].im);
@@ -220,10 +240,9 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
         __syncthreads();
         if (live) {
             // A_pp^-1 D_pq|_B t (p-site i)
-            block_hops<LF>(p, sp_, pp, Tq, vbh, ht, acc);
+            block_hops<LF>(p, sp_, i, pp, Tq, vbh, ht, acc);
             clover_inv_apply(static_cast<const float4 *>(p.clov[pp][grp]), Vh, sp_.s, acc);
         }
-        __syncthreads();  // every t read: T now holds q
         float d[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // <q, rho> re, im per lane; |q|^2 per lane
         if (live) {
             // q = rho - A_pp^-1 D_pq|_B t
@@ -233,7 +252,7 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
                 const ulonglong2 rv = R[k * vbh + i];
                 const C2 rho = {rv.x, rv.y};
                 const C2 q = c2_sub(rho, acc[k]);
-                Tq[k * vbh + i] = make_ulonglong2(q.re, q.im);
+                acc[k] = q;
                 dre = ffma2(q.re, rho.re, dre);
                 dre = ffma2(q.im, rho.im, dre);
                 dim = ffma2(q.re, rho.im, dim);
@@ -256,12 +275,11 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
             const C2 mom = {fneg2(om.re), fneg2(om.im)};
 #pragma unroll
             for (int k = 0; k < 12; k++) {
-                const ulonglong2 rv = R[k * vbh + i], qv = Tq[k * vbh + i], dv = D[k * vbh + i];
-                C2 rho = {rv.x, rv.y};
-                const C2 dl = c2_lanefma(om, rho, C2{dv.x, dv.y});
-                rho = c2_lanefma(mom, C2{qv.x, qv.y}, rho);
-                R[k * vbh + i] = make_ulonglong2(rho.re, rho.im);
-                D[k * vbh + i] = make_ulonglong2(dl.re, dl.im);
+                const ulonglong2 rv = R[k * vbh + i];
+                const C2 rho = {rv.x, rv.y};
+                D[k] = c2_lanefma(om, rho, D[k]);
+                const C2 left = c2_lanefma(mom, acc[k], rho);
+                R[k * vbh + i] = make_ulonglong2(left.re, left.im);
             }
         }
     }
@@ -269,14 +287,14 @@ __global__ void __launch_bounds__(128, 3) k_sap_block(const SapParams p)
         ulonglong2 *z = static_cast<ulonglong2 *>(p.z) + sp_.s * P + q0;
 #pragma unroll
         for (int k = 0; k < 12; k++) {
-            const ulonglong2 zv = z[k * cs], dv = D[k * vbh + i];
-            const C2 s = c2_add({zv.x, zv.y}, C2{dv.x, dv.y});
+            const ulonglong2 zv = z[k * cs];
+            const C2 s = c2_add({zv.x, zv.y}, D[k]);
             z[k * cs] = make_ulonglong2(s.re, s.im);
         }
     }
 }
 
-// 4^4 blocks need 72 KB of dynamic shared memory plus the reduction scratch:
+// 4^4 blocks need 48 KB of dynamic shared memory plus the reduction scratch:
 // opt in once per kernel
 template <int LF>
 cudaError_t launch_sap_k(const SapParams &p, dim3 grid, int threads, size_t smem, cudaStream_t st)
@@ -306,7 +324,7 @@ cudaError_t launch_sap_block(const SapParams &p, int link_fmt, cudaStream_t st)
     const int vbh = p.bs[0] * p.bs[1] * p.bs[2] * p.bs[3] / 2;
     if (vbh < 1 || vbh > 128 || p.nrhs % 2) return cudaErrorInvalidValue;
     const int threads = (vbh + 31) / 32 * 32;
-    const size_t smem = (size_t)3 * 12 * vbh * sizeof(ulonglong2);
+    const size_t smem = (size_t)2 * 12 * vbh * sizeof(ulonglong2);
     const int nbt = p.nb[0] * p.nb[1] * p.nb[2] * p.nb[3];
     dim3 grid(p.nrhs / 2, p.nb[1] % 2 == 0 ? nbt / 2 : nbt);
     switch (link_fmt) {

@@ -61,7 +61,7 @@ __device__ __forceinline__ double snorm(const V12 &a)
          s += (long long)gridDim.x * c.lanes)
 
 // p = r + beta (p - omega v); first iteration p = r
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_p(Cfg c, const void *rv, void *pv, const void *vv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_p(Cfg c, const void *rv, void *pv, const void *vv, long long Vh, int nrhs,
                          const RhsState *st, int first)
 {
     SITE_LOOP
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_p(Cfg c, const void *rv, voi
 }
 
 // alpha = rho / <rhat, v>
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_alpha(Cfg c, const void *rh, const void *vv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_alpha(Cfg c, const void *rh, const void *vv, long long Vh, int nrhs,
                              RhsState *st, double *partials, unsigned int *counter)
 {
     double acc[2] = {0, 0};
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_alpha(Cfg c, const void *rh,
 }
 
 // s = r - alpha v
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_s(Cfg c, const void *rv, const void *vv, void *sv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_s(Cfg c, const void *rv, const void *vv, void *sv, long long Vh, int nrhs,
                          const RhsState *st)
 {
     SITE_LOOP
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_s(Cfg c, const void *rv, con
 }
 
 // omega = <t, s> / <t, t>
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_omega(Cfg c, const void *tv, const void *sv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_omega(Cfg c, const void *tv, const void *sv, long long Vh, int nrhs,
                              RhsState *st, double *partials, unsigned int *counter)
 {
     double acc[3] = {0, 0, 0};
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_omega(Cfg c, const void *tv,
 }
 
 // x += alpha p + omega s; r = s - omega t; rho' = <rhat, r>; |r|^2
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_update(Cfg c, void *xv, void *rv, const void *pv, const void *sv,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_update(Cfg c, void *xv, void *rv, const void *pv, const void *sv,
                               const void *tv, const void *rh, long long Vh, int nrhs,
                               RhsState *st, int max_iter, double *partials, unsigned int *counter, int *n_active)
 {
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_update(Cfg c, void *xv, void
 }
 
 // inner init: r = b, rhat = r (b may alias rhat); rho = |r|^2, tol2 *= |r|^2
-__global__ void __launch_bounds__(kMaxBlock) k_bicg_init(Cfg c, const void *bv, void *rv, void *rh, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_bicg_init(Cfg c, const void *bv, void *rv, void *rh, long long Vh, int nrhs,
                             RhsState *st, double *partials, unsigned int *counter, int *n_active)
 {
     double acc[1] = {0};
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_bicg_init(Cfg c, const void *bv, 
 // ---- CGNE on the normal equations (real per-RHS scalars) ----
 
 // rho' = |z|^2, beta = rho'/rho
-__global__ void __launch_bounds__(kMaxBlock) k_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs,
                                                         RhsState *st, int first, double *partials,
                                                         unsigned int *counter)
 {
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_gamma(Cfg c, const void *zv, l
 }
 
 // p = z + beta p
-__global__ void __launch_bounds__(kMaxBlock) k_cg_p(Cfg c, const void *zv, void *pv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_cg_p(Cfg c, const void *zv, void *pv, long long Vh, int nrhs,
                                                     const RhsState *st)
 {
     SITE_LOOP
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_p(Cfg c, const void *zv, void 
 }
 
 // alpha = rho / |w|^2
-__global__ void __launch_bounds__(kMaxBlock) k_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs,
                                                         RhsState *st, double *partials,
                                                         unsigned int *counter)
 {
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_alpha(Cfg c, const void *wv, l
 }
 
 // x += alpha p, r -= alpha w, |r|^2
-__global__ void __launch_bounds__(kMaxBlock) k_cg_update(Cfg c, void *xv, void *rv, const void *pv,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_cg_update(Cfg c, void *xv, void *rv, const void *pv,
                                                          const void *wv, long long Vh, int nrhs,
                                                          RhsState *st, int max_iter, double *partials,
                                                          unsigned int *counter, int *n_active)
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_cg_update(Cfg c, void *xv, void *
 // FP64 outer residual r = b - y and |r|^2; an RHS flagged `fresh` (x = 0)
 // takes r = b and also records |b|^2, turning tol2 = r_target^2 into the
 // absolute threshold r_target^2 |b|^2
-__global__ void __launch_bounds__(kMaxBlock) k_residual64(Cfg c, const double2 *b, const double2 *y, double2 *rv,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_residual64(Cfg c, const double2 *b, const double2 *y, double2 *rv,
                              long long Vh, int nrhs, RhsState *st, const int *mask,
                              double *partials, unsigned int *counter, int *n_active)
 {
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_residual64(Cfg c, const double2 *
     count_active(st, nrhs, n_active);
 }
 
-__global__ void __launch_bounds__(kMaxBlock) k_norm2(Cfg c, const double2 *v, long long Vh, int nrhs, double *out,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_norm2(Cfg c, const double2 *v, long long Vh, int nrhs, double *out,
                         double *partials, unsigned int *counter)
 {
     double acc[1] = {0};
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kMaxBlock) k_norm2(Cfg c, const double2 *v, lo
     if ((int)threadIdx.x < nrhs) out[threadIdx.x] = tot[0];
 }
 
-__global__ void __launch_bounds__(kMaxBlock) k_diff_norm2(Cfg c, const double2 *a, const double2 *b, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k_diff_norm2(Cfg c, const double2 *a, const double2 *b, long long Vh, int nrhs,
                              double *out, double *partials, unsigned int *counter)
 {
     double acc[1] = {0};

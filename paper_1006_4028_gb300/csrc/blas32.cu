@@ -1,16 +1,18 @@
 // FP32 inner-solver BLAS-1 kernels on the paired layout of pair.cuh: one
 // thread per (site, RHS pair), every update one packed f32x2 instruction for
 // the two RHS, per-RHS scalars (alpha, omega, beta) held per lane.  Dot
-// products are summed in FP32 over the sites one thread visits (24 terms a
-// site, a few tens of sites: one packed f32x2 add per site and value, where
-// an FP64 add per site would run on GB300's 1/64-rate FP64 pipe) and across
-// threads and blocks on 64-bit integers per RHS; the reductions and the scalar
+// products are summed in FP32 over the 24 terms of a site, compensated over the
+// sites one thread visits (an FP64 add per site would run on GB300's 1/64-rate
+// FP64 pipe) and across threads and blocks on 64-bit integers per RHS; the reductions and the scalar
 // recurrences (those the FP64 kernels share, and the shadow-form BiCGStab's
 // own) are in reduce.cuh, so every decision stays per RHS.
 //
 // A pair is processed while either of its RHS is active; an inactive lane's
 // solution x is never changed (lane blend), and its terms are excluded from
 // every reduction.  Other vectors of an inactive lane are scratch.
+#include <algorithm>
+#include <cmath>
+
 #include "cplx.cuh"
 #include "dp_internal.h"
 #include "pair.cuh"
@@ -18,6 +20,16 @@
 
 namespace dp {
 namespace {
+
+// The passes stream whole fields, bound by HBM (L2 on small lattices).  What
+// keeps the memory busy is loads in flight, and a thread that issues many
+// before it uses one does better than more threads: the launch bounds ask for
+// one block per SM, so up to 128 registers hold them, and the smaller grid
+// also leaves the reduction fewer partials.  Components of a site loaded
+// together in the s and the update pass, measured over 1 to 12:
+// 48x24^3, 12 RHS: s 305 -> 275 us, update 557 -> 497 us (6.9 TB/s);
+// 32x16^3, 48 RHS: 233 -> 178, 394 -> 310; 24x16x12^2, 12 RHS: 42 -> 29, 62 -> 45.
+constexpr int kSBatch = 6, kUBatch = 2;
 
 struct P12 {
     C2 c[12];
@@ -73,11 +85,23 @@ __device__ __forceinline__ f2 pnorm(const P12 &a)
     return s;
 }
 
+// a thread's sum over its sites, compensated (Kahan): its error does not grow
+// with the sites a thread visits, so the grid can be chosen for speed alone
+struct KSum {
+    f2 s = 0ull, c = 0ull;
+    __device__ __forceinline__ void add(f2 x)
+    {
+        const f2 y = fadd2(x, fneg2(c)), t = fadd2(s, y);
+        c = fadd2(fadd2(t, fneg2(s)), fneg2(y));
+        s = t;
+    }
+};
+
 // the two lanes of a thread's sum, zero for an inactive RHS
-__device__ __forceinline__ void set_lanes(float &d0, float &d1, f2 v, bool a0, bool a1)
+__device__ __forceinline__ void set_lanes(float &d0, float &d1, const KSum &v, bool a0, bool a1)
 {
     float l0, l1;
-    upk(v, l0, l1);
+    upk(v.s, l0, l1);
     d0 = a0 ? l0 : 0.f;
     d1 = a1 ? l1 : 0.f;
 }
@@ -94,18 +118,18 @@ __device__ __forceinline__ void set_lanes(float &d0, float &d1, f2 v, bool a0, b
     PAIR_VARS;                                                                 \
     PAIR_FOR
 
-__global__ void __launch_bounds__(kMaxBlock) k32_alpha(Cfg c, const void *rh, const void *vv, long long Vh, int nrhs,
+__global__ void __launch_bounds__(kMaxBlock, 1) k32_alpha(Cfg c, const void *rh, const void *vv, long long Vh, int nrhs,
                           RhsState *st, double *partials, unsigned int *counter, int *n_active)
 {
     float acc[4];  // RHS 2q: re, im; 2q + 1: re, im
     {
-        f2 sum0 = 0ull, sum1 = 0ull;
+        KSum sum0, sum1;
         PAIR_LOOP
         {
             const long long me = s * P + q;
             const C2 d = pdot(ldp(rh, cs, me), ldp(vv, cs, me));
-            sum0 = fadd2(sum0, d.re);
-            sum1 = fadd2(sum1, d.im);
+            sum0.add(d.re);
+            sum1.add(d.im);
         }
         set_lanes(acc[0], acc[2], sum0, a0, a1);
         set_lanes(acc[1], acc[3], sum1, a0, a1);
@@ -120,13 +144,13 @@ __global__ void __launch_bounds__(kMaxBlock) k32_alpha(Cfg c, const void *rh, co
 // keep the lanes of `old` whose RHS is inactive
 __device__ __forceinline__ f2 blend(f2 nw, f2 old, f2 m) { return (nw & m) | (old & ~m); }
 
-__global__ void __launch_bounds__(kMaxBlock) k32_init(Cfg c, const void *bv, void *rv, void *rh, void *pv,
+__global__ void __launch_bounds__(kMaxBlock, 1) k32_init(Cfg c, const void *bv, void *rv, void *rh, void *pv,
                                                       long long Vh, int nrhs, RhsState *st,
                                                       double *partials, unsigned int *counter, int *n_active)
 {
     float acc[2];
     {
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -134,7 +158,7 @@ __global__ void __launch_bounds__(kMaxBlock) k32_init(Cfg c, const void *bv, voi
             stp(rv, cs, me, b);
             stp(rh, cs, me, b);
             if (pv) stp(pv, cs, me, b);
-            sum0 = fadd2(sum0, pnorm(b));
+            sum0.add(pnorm(b));
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -153,7 +177,7 @@ __global__ void __launch_bounds__(kMaxBlock) k32_init(Cfg c, const void *bv, voi
 // 14 vector streams per iteration (s_dots: r, v, rhat, rhat' -> s; update:
 // x, p, s, t, v, rhat' -> x, r, p) and no separate alpha or omega pass.
 
-__global__ void __launch_bounds__(kMaxBlock) k32_s_dots(Cfg c, const void *rv, const void *vv,
+__global__ void __launch_bounds__(kMaxBlock, 1) k32_s_dots(Cfg c, const void *rv, const void *vv,
                                                         void *sv, const void *rh, const void *rh2,
                                                         long long Vh, int nrhs, RhsState *st,
                                                         double *partials, unsigned int *counter)
@@ -162,32 +186,39 @@ __global__ void __launch_bounds__(kMaxBlock) k32_s_dots(Cfg c, const void *rv, c
     {
         const int qq = threadIdx.x % (nrhs / 2);
         const C2 mal = neg(lanes(st[2 * qq].alpha_f, st[2 * qq + 1].alpha_f));
-        f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull, sum3 = 0ull;
+        KSum sum0, sum1, sum2, sum3;
         PAIR_LOOP
         {
             const long long me = s * P + q;
             f2 rsr = 0ull, rsi = 0ull, rtr = 0ull, rti = 0ull;
-#pragma unroll 4
-            for (int k = 0; k < 12; k++) {
-                // every load ahead of the store (the pointers may alias, so a
-                // later load could not be moved above it)
-                const C2 r = ld1(rv, cs, me, k), v = ld1(vv, cs, me, k);
-                const C2 h = ld1(rh, cs, me, k), h2 = ld1(rh2, cs, me, k);
-                const C2 sx = c2_lanefma(mal, v, r);
-                st1(sv, cs, me, k, sx);
-                rsr = ffma2(h.re, sx.re, rsr);
-                rsr = ffma2(h.im, sx.im, rsr);
-                rsi = ffma2(h.re, sx.im, rsi);
-                rsi = ffma2(fneg2(h.im), sx.re, rsi);
-                rtr = ffma2(h2.re, sx.re, rtr);
-                rtr = ffma2(h2.im, sx.im, rtr);
-                rti = ffma2(h2.re, sx.im, rti);
-                rti = ffma2(fneg2(h2.im), sx.re, rti);
+#pragma unroll 1
+            for (int k0 = 0; k0 < 12; k0 += kSBatch) {
+                C2 r[kSBatch], v[kSBatch], h[kSBatch], h2[kSBatch];
+#pragma unroll
+                for (int i = 0; i < kSBatch; i++) {
+                    r[i] = ld1(rv, cs, me, k0 + i);
+                    v[i] = ld1(vv, cs, me, k0 + i);
+                    h[i] = ld1(rh, cs, me, k0 + i);
+                    h2[i] = ld1(rh2, cs, me, k0 + i);
+                }
+#pragma unroll
+                for (int i = 0; i < kSBatch; i++) {
+                    const C2 sx = c2_lanefma(mal, v[i], r[i]);
+                    st1(sv, cs, me, k0 + i, sx);
+                    rsr = ffma2(h[i].re, sx.re, rsr);
+                    rsr = ffma2(h[i].im, sx.im, rsr);
+                    rsi = ffma2(h[i].re, sx.im, rsi);
+                    rsi = ffma2(fneg2(h[i].im), sx.re, rsi);
+                    rtr = ffma2(h2[i].re, sx.re, rtr);
+                    rtr = ffma2(h2[i].im, sx.im, rtr);
+                    rti = ffma2(h2[i].re, sx.im, rti);
+                    rti = ffma2(fneg2(h2[i].im), sx.re, rti);
+                }
             }
-            sum0 = fadd2(sum0, rsr);
-            sum1 = fadd2(sum1, rsi);
-            sum2 = fadd2(sum2, rtr);
-            sum3 = fadd2(sum3, rti);
+            sum0.add(rsr);
+            sum1.add(rsi);
+            sum2.add(rtr);
+            sum3.add(rti);
         }
         set_lanes(acc[0], acc[4], sum0, a0, a1);
         set_lanes(acc[1], acc[5], sum1, a0, a1);
@@ -200,23 +231,32 @@ __global__ void __launch_bounds__(kMaxBlock) k32_s_dots(Cfg c, const void *rv, c
     if (r < nrhs) finish_s_dots(st[r], v[0], v[1], v[2], v[3]);
 }
 
-__global__ void __launch_bounds__(kMaxBlock) k32_omega_dots(Cfg c, const void *dots, long long Vh,
+__global__ void __launch_bounds__(kMaxBlock, 1) k32_omega_dots(Cfg c, const void *dots, long long Vh,
                                                             int nrhs, RhsState *st,
                                                             double *partials, unsigned int *counter)
 {
     float acc[6];
     {
         const f2 *d = static_cast<const f2 *>(dots);
-        f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull;
+        KSum sum0, sum1, sum2;
         PAIR_VARS;
-        // (three loads an item: four items' in flight)
-#pragma unroll 4
-        PAIR_FOR
-        {
-            const long long me = s * P + q;
-            sum0 = fadd2(sum0, __ldg(d + me));
-            sum1 = fadd2(sum1, __ldg(d + cs + me));
-            sum2 = fadd2(sum2, __ldg(d + 2 * cs + me));
+        // three 8-byte loads an item: eight items' in flight, also at the end
+        constexpr int kItems = 8;
+        const long long step = (long long)gridDim.x * c.lanes;
+        for (long long s0 = (long long)blockIdx.x * c.lanes + lane; (a0 || a1) && s0 < Vh; s0 += kItems * step) {
+            f2 w[kItems][3];
+#pragma unroll
+            for (int i = 0; i < kItems; i++) {
+                const long long s = s0 + i * step;
+#pragma unroll
+                for (int k = 0; k < 3; k++) w[i][k] = s < Vh ? __ldg(d + s * P + q + k * cs) : 0ull;
+            }
+#pragma unroll
+            for (int i = 0; i < kItems; i++) {
+                sum0.add(w[i][0]);
+                sum1.add(w[i][1]);
+                sum2.add(w[i][2]);
+            }
         }
         set_lanes(acc[0], acc[3], sum0, a0, a1);
         set_lanes(acc[1], acc[4], sum1, a0, a1);
@@ -228,7 +268,7 @@ __global__ void __launch_bounds__(kMaxBlock) k32_omega_dots(Cfg c, const void *d
     if (r < nrhs) finish_omega_shadow(st[r], v[0], v[1], v[2]);
 }
 
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_update_pa(Cfg c, void *xv, void *rv, void *pv, const void *sv, const void *tv, const void *vv,
               const void *rh2, long long Vh, int nrhs, RhsState *st, int max_iter,
               double *partials, unsigned int *counter, int *n_active)
@@ -240,35 +280,45 @@ k32_update_pa(Cfg c, void *xv, void *rv, void *pv, const void *sv, const void *t
         const C2 om = lanes(st[2 * qq].omega_f, st[2 * qq + 1].omega_f);
         const C2 be = lanes(st[2 * qq].beta_f, st[2 * qq + 1].beta_f);
         const C2 mom = neg(om);
-        f2 sum0 = 0ull, sum1 = 0ull, sum2 = 0ull;
+        KSum sum0, sum1, sum2;
         PAIR_LOOP
         {
             const long long me = s * P + q;
             const f2 m = (a0 ? 0x00000000ffffffffull : 0ull) | (a1 ? 0xffffffff00000000ull : 0ull);
             f2 nn = 0ull, rpr = 0ull, rpi = 0ull;
-#pragma unroll 4
-            for (int k = 0; k < 12; k++) {
-                const C2 x = ld1(xv, cs, me, k), p = ld1(pv, cs, me, k), sx = ld1(sv, cs, me, k);
-                const C2 t = ld1(tv, cs, me, k), v = ld1(vv, cs, me, k);
-                const C2 h2 = ld1(rh2, cs, me, k);  // with the others, ahead of the stores
-                C2 xn = c2_lanefma(om, sx, c2_lanefma(al, p, x));
-                xn.re = blend(xn.re, x.re, m);
-                xn.im = blend(xn.im, x.im, m);
-                st1(xv, cs, me, k, xn);
-                const C2 r = c2_lanefma(mom, t, sx);
-                st1(rv, cs, me, k, r);
-                const C2 pn = c2_lanefma(be, c2_lanefma(mom, v, p), r);
-                st1(pv, cs, me, k, pn);
-                nn = ffma2(r.re, r.re, nn);
-                nn = ffma2(r.im, r.im, nn);
-                rpr = ffma2(h2.re, pn.re, rpr);
-                rpr = ffma2(h2.im, pn.im, rpr);
-                rpi = ffma2(h2.re, pn.im, rpi);
-                rpi = ffma2(fneg2(h2.im), pn.re, rpi);
+#pragma unroll 1
+            for (int k0 = 0; k0 < 12; k0 += kUBatch) {
+                C2 x[kUBatch], p[kUBatch], sx[kUBatch], t[kUBatch], v[kUBatch], h2[kUBatch];
+#pragma unroll
+                for (int i = 0; i < kUBatch; i++) {
+                    x[i] = ld1(xv, cs, me, k0 + i);
+                    p[i] = ld1(pv, cs, me, k0 + i);
+                    sx[i] = ld1(sv, cs, me, k0 + i);
+                    t[i] = ld1(tv, cs, me, k0 + i);
+                    v[i] = ld1(vv, cs, me, k0 + i);
+                    h2[i] = ld1(rh2, cs, me, k0 + i);
+                }
+#pragma unroll
+                for (int i = 0; i < kUBatch; i++) {
+                    C2 xn = c2_lanefma(om, sx[i], c2_lanefma(al, p[i], x[i]));
+                    xn.re = blend(xn.re, x[i].re, m);
+                    xn.im = blend(xn.im, x[i].im, m);
+                    st1(xv, cs, me, k0 + i, xn);
+                    const C2 r = c2_lanefma(mom, t[i], sx[i]);
+                    st1(rv, cs, me, k0 + i, r);
+                    const C2 pn = c2_lanefma(be, c2_lanefma(mom, v[i], p[i]), r);
+                    st1(pv, cs, me, k0 + i, pn);
+                    nn = ffma2(r.re, r.re, nn);
+                    nn = ffma2(r.im, r.im, nn);
+                    rpr = ffma2(h2[i].re, pn.re, rpr);
+                    rpr = ffma2(h2[i].im, pn.im, rpr);
+                    rpi = ffma2(h2[i].re, pn.im, rpi);
+                    rpi = ffma2(fneg2(h2[i].im), pn.re, rpi);
+                }
             }
-            sum0 = fadd2(sum0, nn);
-            sum1 = fadd2(sum1, rpr);
-            sum2 = fadd2(sum2, rpi);
+            sum0.add(nn);
+            sum1.add(rpr);
+            sum2.add(rpi);
         }
         set_lanes(acc[0], acc[3], sum0, a0, a1);
         set_lanes(acc[1], acc[4], sum1, a0, a1);
@@ -290,13 +340,13 @@ k32_update_pa(Cfg c, void *xv, void *rv, void *pv, const void *sv, const void *t
 
 __device__ __forceinline__ f2 lanes_re(float a0, float a1) { return pk(a0, a1); }
 
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs, RhsState *st, int first,
              double *partials, unsigned int *counter)
 {
     float acc[2];
     {
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -307,7 +357,7 @@ k32_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs, RhsState *st, int fi
                 nn = ffma2(z.re, z.re, nn);
                 nn = ffma2(z.im, z.im, nn);
             }
-            sum0 = fadd2(sum0, nn);
+            sum0.add(nn);
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -318,7 +368,7 @@ k32_cg_gamma(Cfg c, const void *zv, long long Vh, int nrhs, RhsState *st, int fi
 }
 
 // p = z + beta p
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_cg_p(Cfg c, const void *zv, void *pv, long long Vh, int nrhs, const RhsState *st)
 {
     const int qq = threadIdx.x % (nrhs / 2);
@@ -338,13 +388,13 @@ k32_cg_p(Cfg c, const void *zv, void *pv, long long Vh, int nrhs, const RhsState
 }
 
 // alpha = rho / |w|^2
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs, RhsState *st, double *partials,
              unsigned int *counter)
 {
     float acc[2];
     {
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -355,7 +405,7 @@ k32_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs, RhsState *st, double
                 nn = ffma2(w.re, w.re, nn);
                 nn = ffma2(w.im, w.im, nn);
             }
-            sum0 = fadd2(sum0, nn);
+            sum0.add(nn);
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -366,7 +416,7 @@ k32_cg_alpha(Cfg c, const void *wv, long long Vh, int nrhs, RhsState *st, double
 }
 
 // x += alpha p (active lanes only), r -= alpha w, |r|^2
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long long Vh, int nrhs,
               RhsState *st, int max_iter, double *partials, unsigned int *counter, int *n_active)
 {
@@ -375,7 +425,7 @@ k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long lo
         const int qq = threadIdx.x % (nrhs / 2);
         const f2 al = lanes_re(st[2 * qq].alpha_f.x, st[2 * qq + 1].alpha_f.x);
         const f2 mal = fneg2(al);
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -396,7 +446,7 @@ k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long lo
                 nn = ffma2(r.re, r.re, nn);
                 nn = ffma2(r.im, r.im, nn);
             }
-            sum0 = fadd2(sum0, nn);
+            sum0.add(nn);
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -411,13 +461,13 @@ k32_cg_update(Cfg c, void *xv, void *rv, const void *pv, const void *wv, long lo
 // arrays, and updates with per-RHS coefficients read from them ----
 
 // out[r] = <a, b> = sum conj(a) b (complex) per RHS
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_dotv(Cfg c, const void *av, const void *bv, long long Vh, int nrhs, const RhsState *st,
          double2 *out, double *partials, unsigned int *counter)
 {
     float acc[4];
     {
-        f2 sum0 = 0ull, sum1 = 0ull;
+        KSum sum0, sum1;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -430,8 +480,8 @@ k32_dotv(Cfg c, const void *av, const void *bv, long long Vh, int nrhs, const Rh
                 im = ffma2(x.re, y.im, im);
                 im = ffma2(fneg2(x.im), y.re, im);
             }
-            sum0 = fadd2(sum0, re);
-            sum1 = fadd2(sum1, im);
+            sum0.add(re);
+            sum1.add(im);
         }
         set_lanes(acc[0], acc[2], sum0, a0, a1);
         set_lanes(acc[1], acc[3], sum1, a0, a1);
@@ -443,13 +493,13 @@ k32_dotv(Cfg c, const void *av, const void *bv, long long Vh, int nrhs, const Rh
 }
 
 // out[r] = |a|^2 per RHS
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_norm2v(Cfg c, const void *av, long long Vh, int nrhs, const RhsState *st, double *out,
            double *partials, unsigned int *counter)
 {
     float acc[2];
     {
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -460,7 +510,7 @@ k32_norm2v(Cfg c, const void *av, long long Vh, int nrhs, const RhsState *st, do
                 nn = ffma2(x.re, x.re, nn);
                 nn = ffma2(x.im, x.im, nn);
             }
-            sum0 = fadd2(sum0, nn);
+            sum0.add(nn);
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -477,7 +527,7 @@ __device__ __forceinline__ C2 coef_lanes(const double2 *cf, int q, double sign)
 }
 
 // w -= c wi, z -= c zi (modified Gram-Schmidt step, c per RHS)
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_mgs(Cfg c, void *wv, void *zv, const void *wiv, const void *ziv, long long Vh, int nrhs,
         const RhsState *st, const double2 *cf)
 {
@@ -495,7 +545,7 @@ k32_mgs(Cfg c, void *wv, void *zv, const void *wiv, const void *ziv, long long V
 }
 
 // w /= |w|, z /= |w| (nrm = |w|^2 per RHS)
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_normalise(Cfg c, void *wv, void *zv, long long Vh, int nrhs, const RhsState *st,
               const double *nrm)
 {
@@ -517,7 +567,7 @@ k32_normalise(Cfg c, void *wv, void *zv, long long Vh, int nrhs, const RhsState 
 }
 
 // x += a z (active lanes), r -= a w, |r|^2 -> convergence (a = <w, r> per RHS)
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
 k32_gcr_update(Cfg c, void *xv, void *rv, const void *zv, const void *wv, long long Vh, int nrhs,
                RhsState *st, const double2 *cf, int max_iter, double *partials,
                unsigned int *counter, int *n_active)
@@ -526,7 +576,7 @@ k32_gcr_update(Cfg c, void *xv, void *rv, const void *zv, const void *wv, long l
     {
         const int qq = threadIdx.x % (nrhs / 2);
         const C2 a = coef_lanes(cf, qq, 1.0), ma = coef_lanes(cf, qq, -1.0);
-        f2 sum0 = 0ull;
+        KSum sum0;
         PAIR_LOOP
         {
             const long long me = s * P + q;
@@ -544,7 +594,7 @@ k32_gcr_update(Cfg c, void *xv, void *rv, const void *zv, const void *wv, long l
                 nn = ffma2(r.re, r.re, nn);
                 nn = ffma2(r.im, r.im, nn);
             }
-            sum0 = fadd2(sum0, nn);
+            sum0.add(nn);
         }
         set_lanes(acc[0], acc[1], sum0, a0, a1);
     }
@@ -642,7 +692,11 @@ cudaError_t blas32_omega_dots(BlasCtx &bc, const void *dots, long long Vh, int n
                               cudaStream_t s)
 {
     if (nrhs % 2) return cudaErrorInvalidValue;
-    const Cfg c = cfg_wave(bc, k32_omega_dots, Vh, nrhs / 2);
+    Cfg c = cfg_wave(bc, k32_omega_dots, Vh, nrhs / 2);
+    // 24 bytes an item: what counts is the rounds of eight loads, Vh / (8 lanes
+    // grid) in the blocks and 6 grid / (8 lanes) in the last one, fewest near
+    // grid = sqrt(Vh) / 2 (32x16^3, 48 RHS: 304 blocks 41 us, 128 blocks 21)
+    c.grid = std::min(c.grid, std::max(c.lanes, (int)std::sqrt((double)Vh) / 2));
     k32_omega_dots<<<c.grid, c.block, 0, s>>>(c, dots, Vh, nrhs, st, bc.partials, bc.counter);
     return cudaGetLastError();
 }

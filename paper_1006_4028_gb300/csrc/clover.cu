@@ -346,7 +346,7 @@ __global__ void k_clover_point64(const CloverApplyParams p, Geom g, const SlotIn
 // Per-RHS |(mat + diag) in|^2 of an FP64 spinor with an FP32 clover (mat),
 // the product formed in FP32 and the squares summed in FP64: a residual
 // report needs a few digits only.  Block = lanes x n RHS (reduce.cuh).
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
     k_clover_norm(Cfg c, const CloverApplyParams p, double *out, double *partials,
                   unsigned int *counter)
 {

@@ -3,7 +3,7 @@
 // A block is `lanes` sites x `units` threads, thread t = lane*units + unit;
 // a unit is one RHS (FP64) or one RHS pair (FP32 paired layout, LANES = 2).
 // Each thread passes per-RHS partial sums; the block sums them over its
-// lanes in a fixed tree, writes one partial per RHS to global scratch, and
+// lanes in a fixed order, writes one partial per RHS to global scratch, and
 // the last block to finish (atomic ticket) sums the block partials in a fixed
 // order.  The result for an RHS never depends on the other RHS.
 //
@@ -12,8 +12,8 @@
 // 384-thread block with 8 values a thread, the last block's pass over 300
 // partials and the FP64 conversions around them took most of a reduction
 // kernel on a small lattice (16x8^3, 12 RHS: the three of a BiCGStab iteration
-// 20, 17 and 16 us, now 16, 13 and 10).  An integer add with alignment is
-// about 10 instructions.  Terms are aligned to the largest
+// 20, 17 and 16 us, with integers 16, 13 and 10).  An integer add with
+// alignment is about 10 instructions.  Terms are aligned to the largest
 // one with its leading bit at 2^kLead or above, so a sum of N terms is off by
 // at most N 2^-kLead of its largest term (FP64 adds: N 2^-53 of the sum).
 #pragma once
@@ -343,30 +343,14 @@ __device__ __forceinline__ void finish_cg_update(RhsState &S, double rr, int max
 // true in the threads of the last block; its thread r (r < the RHS count) then
 // has the totals of RHS r in `tot`, so the scalar recurrences of all RHS run
 // side by side in one or two warps.
-
-// sum over the lanes of a block: one barrier a level, the levels taking turns
-// between two regions of `sh`; the result is in the threads of lane 0
-template <int W>
-__device__ __forceinline__ void block_tree(Sum (&v)[W], long long *shm, int *she, const Cfg c, int t, int units,
-                                           int lane)
-{
-    constexpr int kHalf = kMaxBlock / 2;
-    int region = 0;
-    for (int w = c.lanes / 2; w > 0; w >>= 1, region ^= 1) {
-        const int base = region ? kHalf * W : 0;
-        if (lane >= w && lane < 2 * w)
-#pragma unroll
-            for (int k = 0; k < W; k++) {
-                shm[base + (t - w * units) + k * w * units] = v[k].m;
-                she[base + (t - w * units) + k * w * units] = v[k].e;
-            }
-        __syncthreads();
-        if (lane < w)
-#pragma unroll
-            for (int k = 0; k < W; k++)
-                v[k] = add(v[k], Sum{shm[base + t + k * w * units], she[base + t + k * w * units]});
-    }
-}
+//
+// In both passes thread g*n + j sums value j of the n = W*units values over
+// every G-th lane (or block) from g, and thread j then the G results: the
+// W*lanes additions spread over all threads, two barriers a pass.  A tree over
+// the lanes leaves its threads W additions a level, six levels at 12 RHS, and
+// six barriers: the three reductions of an iteration at 16x8^3, 12 RHS, took
+// 16, 13 and 10 us with it and take 11, 7 and 7.
+// n <= the block: cfg_for leaves lanes >= W for every RHS count.
 
 struct __align__(16) Partial {
     long long m;
@@ -374,64 +358,89 @@ struct __align__(16) Partial {
 };
 static_assert(sizeof(Partial) == 16, "two doubles of the scratch each");
 
+// the G sums of each value, left by thread g*n + j at [g*n + j]: thread j's total
+struct GroupSums {
+    long long m[kMaxBlock];
+    int e[kMaxBlock];
+    __device__ __forceinline__ void put(int t, Sum s)
+    {
+        m[t] = s.m;
+        e[t] = s.e;
+    }
+    __device__ __forceinline__ Sum total(int j, int n, int groups) const
+    {
+        Sum s{m[j], e[j]};
+        for (int g = 1; g < groups; g++) s = add(s, Sum{m[g * n + j], e[g * n + j]});
+        return s;
+    }
+};
+
 template <int NV, int LANES, typename T>
 __device__ __forceinline__ bool reduce_last(const T (&in)[LANES * NV], const Cfg c, double *partials,
                                             unsigned int *counter, int units, double (&tot)[NV])
 {
     static_assert(2 * NV <= kRedWidth, "per-RHS partials hold kRedWidth doubles");
     constexpr int W = LANES * NV;
-    __shared__ long long shm[(kMaxBlock / 2 + kMaxBlock / 4) * W];
-    __shared__ int she[(kMaxBlock / 2 + kMaxBlock / 4) * W];
+    __shared__ T raw[W * (kMaxBlock + kMaxRhs / LANES)];
+    __shared__ GroupSums gs;
+    __shared__ double val[W * (kMaxRhs / LANES)];
     __shared__ bool last;
-    const int t = threadIdx.x, u = t % units, lane = t / units;
+    const int t = threadIdx.x;
+    const int n = W * units, grp = t / n, j = t - grp * n, groups = c.block / n;
     Partial *part = reinterpret_cast<Partial *>(partials);
     constexpr int kStride = kMaxRhs * kRedWidth / 2;  // per block
-    const int lead2 = lead_for((int)gridDim.x);
-    {
-        const int lead1 = lead_for(c.lanes);
-        Sum v[W];
+    // value j = k*units + u of lane l at j + l*units + k*block: no bank conflicts
+    const int ld = c.block + units;
 #pragma unroll
-        for (int k = 0; k < W; k++) v[k] = sum_of(in[k], lead1);
-        block_tree<W>(v, shm, she, c, t, units, lane);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < W; k++) {
-                const Sum s = cap(v[k], lead2);
-                part[(long long)blockIdx.x * kStride + (LANES * u + k / NV) * (kRedWidth / 2) + k % NV] =
-                    Partial{s.m, s.e, 0};
-            }
-    }
-    __threadfence();
+    for (int k = 0; k < W; k++) raw[k * ld + t] = in[k];
     __syncthreads();
-    if (t == 0) last = (atomicAdd(counter, 1u) == (unsigned)(gridDim.x - 1));
+    if (grp < groups) {
+        const int lead = lead_for(c.lanes), k = j / units;
+        const T *mine = raw + j + k * c.block;
+        Sum s{0, kSumZero};
+#pragma unroll 4
+        for (int l = grp; l < c.lanes; l += groups) s = add(s, sum_of(mine[l * units], lead));
+        gs.put(t, s);
+    }
+    __syncthreads();
+    if (t < n) {
+        const Sum s = cap(gs.total(t, n, groups), lead_for((int)gridDim.x));
+        part[(long long)blockIdx.x * kStride + t] = Partial{s.m, s.e, 0};
+        __threadfence();
+    }
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
+        last = (atomicAdd(counter, 1u) == (unsigned)(gridDim.x - 1));
+    }
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    // last block: lane l sums blocks l, l+lanes, ... in order, then a fixed tree
-    Sum acc[W];
+    if (grp < groups) {
+        Sum s{0, kSumZero};
+        // eight loads ahead, also at the end (each round waits for L2, about 1 us)
+        constexpr int kAhead = 8;
+        for (int b0 = grp; b0 < (int)gridDim.x; b0 += kAhead * groups) {
+            longlong2 w[kAhead];
 #pragma unroll
-    for (int k = 0; k < W; k++) acc[k] = Sum{0, kSumZero};
-#pragma unroll 4
-    for (int b = lane; b < (int)gridDim.x; b += c.lanes)
+            for (int i = 0; i < kAhead; i++) {
+                const int b = b0 + i * groups;
+                w[i] = make_longlong2(0, kSumZero);
+                if (b < (int)gridDim.x)
+                    w[i] = __ldcg(reinterpret_cast<const longlong2 *>(part + (long long)b * kStride + j));
+            }
 #pragma unroll
-        for (int k = 0; k < W; k++) {
-            const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(
-                part + (long long)b * kStride + (LANES * u + k / NV) * (kRedWidth / 2) + k % NV));
-            acc[k] = add(acc[k], Sum{w.x, (int)w.y});
+            for (int i = 0; i < kAhead; i++) s = add(s, Sum{w[i].x, (int)w[i].y});
         }
-    block_tree<W>(acc, shm, she, c, t, units, lane);
+        gs.put(t, s);
+    }
     if (t == 0) *counter = 0u;
     __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < W; k++) {
-            shm[(LANES * u + k / NV) * NV + k % NV] = acc[k].m;
-            she[(LANES * u + k / NV) * NV + k % NV] = acc[k].e;
-        }
+    if (t < n) val[t] = value(gs.total(t, n, groups));
     __syncthreads();
     if (t < LANES * units)
 #pragma unroll
-        for (int k = 0; k < NV; k++) tot[k] = value(Sum{shm[t * NV + k], she[t * NV + k]});
+        for (int k = 0; k < NV; k++) tot[k] = val[(t % LANES * NV + k) * units + t / LANES];
     return true;
 }
 

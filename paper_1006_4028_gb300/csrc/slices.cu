@@ -130,7 +130,7 @@ __global__ void k_slice_norms_final(const double *partials, int P, int T, int ng
 __device__ __forceinline__ bool refined(const RhsState &S) { return S.active && S.refine; }
 
 // per-RHS |R r|^2 over the refined RHS, thread layout lanes x n (reduce.cuh)
-__global__ void __launch_bounds__(kMaxBlock)
+__global__ void __launch_bounds__(kMaxBlock, 1)
     k_ratio_norm(Cfg c, const double2 *rv, Geom g, int parity, int n, const double *a_out,
                  const double *a_in, const SlotInfo *slots, RhsState *st, double *partials,
                  unsigned int *counter)

@@ -297,12 +297,17 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
     SiteIx *ix = reinterpret_cast<SiteIx *>(smem);
     int4 *buf = smem + spb * (int)(sizeof(SiteIx) / sizeof(int4));
     __shared__ int cmax[kFxBlock];  // largest magnitude (high word) per (group of the launch, site)
+    // the groups with a live RHS: an idle group's clover pointer may be that of
+    // an inverse freed since its job ended
+    __shared__ unsigned groups;
+    if (threadIdx.x == 0) groups = 0;
     const i64 s0 = (i64)blockIdx.x * spb;
     const int ns = (int)min((i64)spb, Vh - s0);
     const int j = threadIdx.x / n, r = threadIdx.x - j * n;
     const i64 s = s0 + j;
     const bool live = j < ns && (!p.active || p.active[r * p.active_stride]);
     if (!__syncthreads_or(live)) return;  // (converged RHS fill the block)
+    if (live) atomicOr(&groups, 1u << fl.of[r]);  // (barriers before its first use)
     for (int k = threadIdx.x; k < ns; k += blockDim.x) {
         const Nbr nb = neighbours(g, s0 + k, p.parity);
         SiteIx q;
@@ -432,6 +437,7 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
         for (int k = threadIdx.x; k < fl.ngrp * ns; k += blockDim.x) cmax[k] = 0;
         __syncthreads();
         for (int gi = 0; gi < fl.ngrp; gi++) {
+            if (!(groups >> gi & 1)) continue;
             const double2 *cl = static_cast<const double2 *>(p.clov[fl.grp[gi]]) + (i64)18 * blk * Vh + s0 + j0;
             unsigned mx = 0;
             for (int e = e0; e < 18; e += es) {
@@ -442,6 +448,7 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
         }
         __syncthreads();
         for (int gi = 0; gi < fl.ngrp; gi++) {
+            if (!(groups >> gi & 1)) continue;
             const double2 *cl = static_cast<const double2 *>(p.clov[fl.grp[gi]]) + (i64)18 * blk * Vh + s0 + j0;
             const int base = max((cmax[gi * ns + j0] >> 20) + 1, 64);
             for (int e = e0; e < 18; e += es) {

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kSliceThreads)
                 const double *w3 = iw + m * 3 * g.Lmax;
                 const double w = w3[g.Lmax + y] * w3[2 * g.Lmax + z] * w3[x];
                 double s2;
-                if (weight_ok(w) && norm2_int(c[par], s2)) {
+                if (norm2_int(c[par], w, s2)) {
                     sum[0] = fmx(s2, w, sum[0]);
                     continue;
                 }

@@ -18,19 +18,24 @@
 
 namespace dp {
 
-// sum of the squares of 24 doubles.  With the leading bit of the largest at
-// bit 59, |v| = hi 2^32 + lo 2: hi hi and hi lo summed in 64 bits, lo lo to 2^34
-// (all of them below 2^-57 of the sum).  false: a value of the largest
-// component's size that the squares (or a product with the weights) could
-// leave the normal range with, an infinity or a NaN
-__device__ __forceinline__ bool norm2_int(const double2 (&v)[12], double &s)
+// sum of the squares of 24 doubles, to be multiplied by the weight w >= 0 and
+// added up over the slice.  With the leading bit of the largest at bit 59, |v|
+// = hi 2^32 + lo 2: hi hi and hi lo summed in 64 bits, lo lo to 2^34 (all of
+// them below 2^-57 of the sum).  false (general arithmetic, which scales each
+// component by 1/alpha first): an infinity or a NaN, a largest component or a
+// weight outside 2^+-400 (squares stay below 2^805), or a product outside
+// 2^+-900: with 1/alpha_t^2 still to come it could leave the normal range
+// although the scaled sum does not (alpha_t = 2^520 and 2^-50 in each space
+// direction: 2^740 times 2^300).  2^900 leaves room for 2^120 terms.
+__device__ __forceinline__ bool norm2_int(const double2 (&v)[12], double w, double &s)
 {
     unsigned mx = 0;
 #pragma unroll
     for (int k = 0; k < 12; k++)
         mx = max(mx, max((unsigned)__double2hiint(v[k].x) & 0x7fffffffu, (unsigned)__double2hiint(v[k].y) & 0x7fffffffu));
-    const int em = (int)(mx >> 20);
-    if (em < 623 || em > 1423) return false;
+    const int em = (int)(mx >> 20), ew = __double2hiint(w) >> 20;
+    if (em < 623 || em > 1423 || ew < 623 || ew > 1423) return false;
+    if (abs(2 * em + ew - 3 * 1023) > 900) return false;
     unsigned long long hh = 0, hl = 0;
     auto sq = [&](double x) {
         const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
@@ -83,19 +88,19 @@ __device__ __forceinline__ SliceShare slice_share(const Geom &g, int r0, int nr)
     return h;
 }
 
-// iw[(m*3 + {0: x, 1: y, 2: z})*Lmax + coordinate] = 1/alpha^2 of group m
+// iw[(m*3 + {0: x, 1: y, 2: z})*Lmax + coordinate] = 1/alpha^2 of group m; 0
+// (a weight that norm2_int refuses) where alpha is outside 2^+-170, so that no
+// product of three, nor of two, rounds among the subnormals
 __device__ __forceinline__ void slice_weights(double *iw, const Geom &g, const double *alpha, int ng)
 {
     for (int k = threadIdx.x; k < ng * 3 * g.Lmax; k += blockDim.x) {
         const int m = k / (3 * g.Lmax), rest = k - m * 3 * g.Lmax;
         const double a = alpha[(long long)m * 4 * g.Lmax + g.Lmax + rest];
-        iw[k] = 1.0 / (a * a);
+        const double w = 1.0 / (a * a);
+        iw[k] = w > 0x1p-340 && w < 0x1p+340 ? w : 0.0;
     }
     __syncthreads();
 }
-
-// a weight that a sum may be multiplied with (else the general arithmetic)
-__device__ __forceinline__ bool weight_ok(double w) { return w > 0x1p-400 && w < 0x1p+400; }
 
 // totals per group over the block: each thread's NV sums are added over the
 // lanes, then over the RHS of a group (grp[r], shared memory) in order; the

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kSliceThreads)
 #pragma unroll
         for (int i = 0; i < 2; i++) {
             double s2;
-            if (INT && weight_ok(w) && norm2_int(c[i], s2)) {
+            if (INT && norm2_int(c[i], w, s2)) {
                 sum[i] = fma(s2, w, sum[i]);
                 continue;
             }

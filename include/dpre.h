@@ -96,6 +96,16 @@ typedef struct {
     const double *table[4]; /* TABLE only: alpha_B,mu per coordinate, length L_mu */
 } dp_profile;
 
+/* The FP64 operator (DP_PREC_FP64 calls, the outer loop of every solve): on
+ * fields whose links are unitary and mix the colours its products run in
+ * integer arithmetic.  A result is off by about 2^-55 of its site's norm, and
+ * each complex component by at most 2^-41 of the sum of its terms' magnitudes
+ * (2^-36 where the inverse clover block has a diagonal entry near a
+ * thirty-second of its largest), whatever stands beside it; chains of FP64
+ * operations leave some 2^-52 of either.  Links that are not unitary, fields of nearly diagonal links
+ * (an entry below 2^-12 in more than one of 500), infinities, NaN and numbers
+ * near the ends of the range take FP64 operations, as does a call or batch
+ * whose scratch for it cannot be had: the bits of a result may then differ. */
 typedef enum {
     DP_PREC_FP64 = 0,       /* FP64 Krylov solve ("FP64 plain" when unbatched)   */
     DP_PREC_MIXED_FP32 = 1, /* FP32 inner BiCGStab, FP32 links, FP64 outer loop  */
@@ -412,7 +422,7 @@ dp_status dp_dslash_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile 
  * (D(alpha_B)^dag = g5 D(1/alpha_B) g5).  These are the operators the BiCGStab
  * and CGNE solvers apply.  in/out: distinct device arrays of one parity in the
  * packed layout of `prec` (see dp_dslash_dev), caller-owned; scratch (two
- * spinor arrays, two hop tables) comes from the context allocator.  FP32 and
+ * spinor arrays, two hop tables, FP64: exponents) comes from the context allocator.  FP32 and
  * 16-bit precisions need nrhs even.  Returns after the stream work finished. */
 dp_status dp_schur_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile *profile,
                        const int src[4], int prec, int compress12, int parity, int dagger,

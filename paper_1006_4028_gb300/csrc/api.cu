@@ -574,7 +574,7 @@ dp_status dp_field_load(dp_ctx *ctx, const double *links, const int dims[4], int
     f->g = g;
     f->bc_t = bc_t;
     double2 *lex = (double2 *)c.alloc(n * sizeof(double));
-    int *flag = (int *)c.alloc(sizeof(int));
+    int *flag = (int *)c.alloc(2 * sizeof(int));
     bool ok = lex != nullptr && flag != nullptr;
     for (int p = 0; p < 2 && ok; p++) {
         f->l64[p] = (double2 *)c.alloc(g.Vh * 4 * 9 * sizeof(double2));
@@ -594,13 +594,13 @@ dp_status dp_field_load(dp_ctx *ctx, const double *links, const int dims[4], int
         return DP_ERR_OOM;
     }
     CUDA_OK(cudaMemcpyAsync(lex, links, n * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-    CUDA_OK(cudaMemsetAsync(flag, 0, sizeof(int), c.stream));
+    CUDA_OK(cudaMemsetAsync(flag, 0, 2 * sizeof(int), c.stream));
     CUDA_OK(launch_pack_links(lex, g, f->l64, f->l32f, f->l32c, flag, c.stream));
     c.launches++;
-    int odd = 0;
-    CUDA_OK(cudaMemcpyAsync(&odd, flag, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    int odd[2] = {0, 0};
+    CUDA_OK(cudaMemcpyAsync(odd, flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     CUDA_OK(cudaStreamSynchronize(c.stream));
-    f->unitary = odd == 0;
+    f->fx = odd[0] == 0 && 500ll * odd[1] <= 4 * g.V;
     c.release(lex);
     c.release(flag);
     std::lock_guard<std::mutex> lk(c.mu);
@@ -744,7 +744,7 @@ dp_status dp_apply(dp_ctx *ctx, dp_field field, int kind, double M, const dp_pro
     void *hopd = c.alloc(hop.size() * sizeof(double));
     // FP64 hops: exponents for the integer kernel (without them the FP64 kernel serves)
     const bool hops = kind == DP_APPLY_HOP || kind == DP_APPLY_FULL;
-    int *ex = hops && pr == 0 && f.unitary ? (int *)c.alloc((size_t)g.V * nk * sizeof(int)) : nullptr;
+    int *ex = hops && pr == 0 && f.fx ? (int *)c.alloc((size_t)g.V * nk * sizeof(int)) : nullptr;
     dp_status ret = DP_OK;
     if (!lex || !ie || !io || !oe || !oo || !te || !to || !hopd) {
         set_error("out of device memory (dp_apply)");
@@ -906,7 +906,7 @@ dp_status dp_dslash_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile 
     // FP64: the integer kernel, with its input's conversion, where its scratch can be had
     void *xw = nullptr;
     int *xe = nullptr;
-    if (pr == 0 && f.unitary) {
+    if (pr == 0 && f.fx) {
         xw = c.alloc((size_t)g.Vh * nrhs * 24 * 8);
         xe = (int *)c.alloc((size_t)g.Vh * nrhs * sizeof(int));
         if (xw && xe) {

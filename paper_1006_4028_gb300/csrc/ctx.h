@@ -37,7 +37,10 @@ struct CloverInv {
 struct Field {
     Geom g;
     int bc_t;
-    bool unitary = false;  // every link's rows have norm 1 (to 1e-3)
+    // FP64 products in integer arithmetic (dslash_fx.cu): every link's rows
+    // and columns have norm 1 (to 1e-3), and at most one link of 500 has an entry below
+    // 2^-12
+    bool fx = false;
     double2 *l64[2] = {nullptr, nullptr};
     float2 *l32f[2] = {nullptr, nullptr};
     float4 *l32c[2] = {nullptr, nullptr};

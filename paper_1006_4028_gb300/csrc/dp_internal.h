@@ -84,7 +84,7 @@ struct DslashParams {
     // BiCGStab omega: f2 (one lane per RHS of a pair) [3][Vh][nrhs/2] holding
     // Re <out, x>, Im <out, x> and |out|^2 over the 12 components of a site
     void *dots;
-    // FP64 in integer arithmetic (dslash_fx.cu; unitary links): NULL, or `in`
+    // FP64 in integer arithmetic (dslash_fx.cu; Field::fx): NULL, or `in`
     // holds fx spinors with these exponents, per (site, RHS) [Vh][nrhs];
     // out_exp (A^-1 epilogue): NULL, or write `out` as fx spinors too
     const int *in_exp;
@@ -172,10 +172,11 @@ cudaError_t launch_clover_norm(BlasCtx &bc, const CloverApplyParams &p, double *
                                cudaStream_t st);
 
 // ---- field packing, sources, restore/contract (field.cu) ----
-// sets *not_unitary (device int, zeroed by the caller) if a row of any link
-// has a squared norm off 1 by more than 1e-3
+// odd (two device ints, zeroed by the caller): [0] is set if a row or a column
+// of any link has a squared norm off 1 by more than 1e-3, [1] counts the links with an
+// entry below 2^-12
 cudaError_t launch_pack_links(const double2 *lex, const Geom &g, double2 *l64[2], float2 *l32f[2],
-                              float4 *l32c[2], int *not_unitary, cudaStream_t st);
+                              float4 *l32c[2], int *odd, cudaStream_t st);
 // lexicographic complex128 spinors [nrhs][V][12] <-> packed parity halves
 cudaError_t launch_pack_spinor(const double2 *lex, const Geom &g, int nrhs, int prec,
                                void *even, void *odd, cudaStream_t st);

@@ -47,7 +47,7 @@
 namespace dp {
 namespace {
 
-// ---- FP64 (scalar): fields whose links are not unitary, or no scratch for dslash_fx.cu ----
+// ---- FP64 (scalar): fields that dslash_fx.cu does not take (Field::fx), or no scratch for it ----
 
 template <int EPI>
 __global__ void __launch_bounds__(256) k_dslash64(const DslashParams p)

@@ -22,16 +22,41 @@
 // accumulators down).  The clover inverse is applied the same way on the
 // renormalised accumulators; the result is rounded to FP64 once, or written as
 // an fx spinor for the next launch.  So a component's error is about 2^-55 of
-// the site's largest one where a chain of FP64 operations leaves about 2^-53.
-// Bounds (rows of U of norm 1, six products a sum): hi hi below 2^59.3, hi lo +
+// the largest one around where a chain of FP64 operations leaves about 2^-53.
+// Bounds (rows and columns of U of norm 1, six products a sum): hi hi below 2^59.3, hi lo +
 // lo hi below 2^62.5, eight directions below 2^62.3; clover (twelve products of
 // anything below 2^59): hi hi below 2^58.6, hi lo + lo hi below 2^62.9.
 //
+// Small components: what FP64 leaves of a component is about 2^-53 of the sum T
+// of its terms' magnitudes.  Where T is near the largest neighbour's size R, as
+// on links that mix the colours, 2^-55 R is less than that; where it is not
+// (links near the unit matrix, one colour much smaller than another) it could
+// be all of a component.  A result with a complex component below 2^-10 R is
+// therefore looked at again (mixes): if some neighbour's projected h is
+// nowhere below 2^-10 R, T is at least that (a row or column of U has norm 1,
+// so its entries' magnitudes add up to 1 or more) and the component is small by
+// cancellation, else the FP64 arithmetic answers.  A spinor with a non-zero
+// component below 2^-16 of its largest is not converted.  So a component is
+// off by at most 2^-41 T (worst case of all truncations: 2^-51 R; 2^-36 T where
+// the inverse clover block has a diagonal entry near a thirty-second of its
+// largest), and a result by 2^-55 of its norm.  On rough links one thread in
+// some 10^5 looks again and the first neighbour answers.  Cost: A^-1 D 540 ->
+// 549 us for 12 RHS on 32x16^3, the FP64 solve there 0.2 % (5 % without the
+// second look).
+//
+// On links that hardly mix the colours a point-source solve falls back often,
+// and a thread alone on the FP64 pipe is slow: 16x8^3, FP64 solve, links exp(i
+// eps H), eps = 0.05 / 0.02 / 0.01 / 0.006: 8.5 / 10.7 / 21 / 23 ms against
+// 7.8 without the guard and 16.7 with k_dslash64.  A field with an entry below
+// 2^-12 in more than one link of 500 (eps below about 0.015; diagonal links)
+// has k_dslash64 throughout (Field::fx).
+//
 // What the integers cannot hold is handed to the FP64 arithmetic, per thread
 // (hop_site64, the code of k_dslash64): a spinor with an infinity or NaN or
-// whose largest component is below 2^-942 or near the overflow threshold is
-// kept as raw doubles (exponent kFxRaw), and its neighbours take that path, as
-// do sites with such entries in the clover block or a result out of range.
+// whose largest component is below 2^-942 or near the overflow threshold, or
+// with a small one as above, is kept as raw doubles (exponent kFxRaw), and its
+// neighbours take that path, as do sites with such entries in the clover block
+// or a result out of range.
 //
 // Why a converted copy: converting in the thread that loads a neighbour (each
 // spinor eight times) cost 13 integer instructions or one 68-cycle cvt per
@@ -124,6 +149,18 @@ __device__ __forceinline__ unsigned top_or(i64 v)
     return (unsigned)(a ^ (a >> 31));
 }
 
+// the smallest of N complex integers, by the high word of its larger part
+template <int N>
+__device__ __forceinline__ unsigned least(const i64 *re, const i64 *im)
+{
+    unsigned m = ~0u;
+#pragma unroll
+    for (int k = 0; k < N; k++) m = min(m, top_or(re[k]) | top_or(im[k]));
+    return m;
+}
+
+constexpr int kSmall = 10;  // results with a component below 2^-kSmall R are looked at again
+constexpr int kKeep = 16;   // spinors with one below 2^-kKeep of the largest are not converted
 constexpr int kMinExp = 81, kMaxExp = 2040;  // biased exponents of the blocks the integers take
 constexpr int kHalf = 1023 + 59;             // value = W 2^(e - kHalf)
 
@@ -286,6 +323,40 @@ __device__ __noinline__ void hop_site64(const DslashParams &p, i64 s, int r)
     hop_site64_body<EPI, true>(p, s, r);
 }
 
+// whether some neighbour's projected h (times its hop factor) has no complex
+// component below 2^-kSmall of the largest neighbour's size, of exponent R
+// (out of line, rare)
+__device__ __noinline__ bool mixes(const DslashParams &p, i64 s, int r, int R)
+{
+    const Geom &g = p.g;
+    const Nbr nb = neighbours(g, s, p.parity);
+    const i64 cs = g.Vh * p.nrhs;
+    const double *ht = static_cast<const double *>(p.hop) + (i64)p.grp_of[r] * 8 * g.Lmax;
+    const int x[4] = {nb.t, nb.x, nb.y, nb.z};
+    bool yes = false;
+#pragma unroll
+    for (int d = 0; d < 8; d++) {
+        if (yes) break;  // (on rough links the first neighbour answers)
+        const int mu = d >> 1;
+        const i64 at = (i64)(d & 1 ? nb.b[mu] : nb.f[mu]) * p.nrhs + r;
+        const unsigned chi = (unsigned)__double2hiint(__ldg(ht + d * g.Lmax + x[mu]));
+        const int e = __ldg(p.in_exp + at) + (int)((chi >> 20) & 0x7ffu) - 1023;
+        const longlong2 *v = static_cast<const longlong2 *>(p.in) + at;
+        const i64 f0 = d & 1 ? -1 : 0, f1 = mu >= 2 ? ~f0 : f0;
+        const int l0 = mu == 1 || mu == 2 ? 9 : 6;  // the lower spin that goes with upper spin 0
+        unsigned m = ~0u;
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const longlong2 a = __ldg(v + k * cs), q = __ldg(v + (k < 3 ? l0 + k : 15 - l0 + k - 3) * cs);
+            const i64 qr = q.x ^ (k < 3 ? f0 : f1), qi = q.y ^ (k < 3 ? f0 : f1);
+            m = min(m, mu & 1 ? top_or(a.x - qi) | top_or(a.y + qr) : top_or(a.x + qr) | top_or(a.y + qi));
+        }
+        // leading bit of the smallest against bit 59
+        yes = m != 0 && e + (63 - __clz((int)m)) - 59 >= R - kSmall;
+    }
+    return yes;
+}
+
 template <int EPI>
 __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
     k_dslash_fx(const __grid_constant__ DslashParams p, const __grid_constant__ FxLaunch fl)
@@ -385,6 +456,8 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
     if (EPI == EPI_HOP || EPI == EPI_XPY || EPI == EPI_XMY_G5) {
         if (live) {
             bool ok = !bad;
+            // (a component of the largest neighbour's size has its leading bit at 56)
+            if (ok && acc.R != kNoExp && !(least<12>(acc.re, acc.im) >> (56 - 32 - kSmall))) ok = mixes(p, s, r, acc.R);
             double2 w[12];
 #pragma unroll
             for (int k = 0; k < 12; k++)  // acc holds -D
@@ -427,12 +500,14 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
             }
         }
     }
-    bool ok = !bad;
+    bool ok = !bad, small = false, hard = false;
     int wexp[2] = {0, 0};
 #pragma unroll
     for (int blk = 0; blk < 2; blk++) {
         // the inverse block of every (group of the launch, site): its largest
-        // exponent, then its limbs (leading bit at 58)
+        // exponent, then its limbs (leading bit at 58); bit 0 of cmax: a diagonal
+        // entry is below 2^-kSmall/2 of the largest, so that its row may add little
+        // of x to the result
         __syncthreads();
         for (int k = threadIdx.x; k < fl.ngrp * ns; k += blockDim.x) cmax[k] = 0;
         __syncthreads();
@@ -444,7 +519,7 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
                 const double2 v = __ldg(cl + (i64)e * Vh);
                 mx = max(mx, max(mag_hi(v.x), mag_hi(v.y)));
             }
-            if (mx) atomicMax(&cmax[gi * ns + j0], (int)mx);
+            if (mx) atomicMax(&cmax[gi * ns + j0], (int)(mx & ~1u));
         }
         __syncthreads();
         for (int gi = 0; gi < fl.ngrp; gi++) {
@@ -455,6 +530,8 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
                 const double2 v = __ldg(cl + (i64)e * Vh);
                 const L2w a = cut31(w59(v.x, base)), b = cut31(w59(v.y, base));
                 buf[(gi * ns + j0) * 18 + e] = make_int4(a.hi, a.lo, b.hi, b.lo);
+                if (e < 3 && min(a.hi < 0 ? -a.hi : a.hi, b.hi < 0 ? -b.hi : b.hi) < 1 << (27 - kSmall / 2))
+                    atomicOr(&cmax[gi * ns + j0], 1);
             }
         }
         __syncthreads();
@@ -510,6 +587,12 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
             acc.im[6 * blk + i] = EPI != EPI_AINV_XMY ? -vi : vi;
         }
         wexp[blk] = we;
+        // (the largest neighbour's size times the block's largest entry: bit 51 + sh)
+        const int low = 51 - 32 - kSmall + sh;
+        if (low > 30 || !(least<6>(acc.re + 6 * blk, acc.im + 6 * blk) >> low)) {
+            small = true;
+            hard = hard || (cmax[gs] & 1);
+        }
         if (EPI == EPI_AINV && p.out_exp) continue;
 #pragma unroll
         for (int k = 6 * blk; k < 6 * blk + 6; k++) {
@@ -522,6 +605,7 @@ __global__ void __launch_bounds__(kFxBlock, 512 / kFxBlock)
         }
     }
     if (!live) return;
+    if (ok && small && acc.R != kNoExp) ok = !hard && mixes(p, s, r, acc.R);
     if (EPI == EPI_AINV && p.out_exp) {
         // an fx spinor: the largest leading bit of the two chiral blocks to bit 59
         int lead = kNoExp;
@@ -567,17 +651,18 @@ __global__ void __launch_bounds__(128) k_to_fx(const double2 *in, longlong2 *w, 
     if (mask && !mask[(int)(gid % n) * stride]) return;
     const i64 cs = Vh * n;
     double2 v[12];
-    unsigned mx = 0, any = 0;
+    unsigned mx = 0, mn = ~0u;  // largest and smallest non-zero complex component
 #pragma unroll
     for (int k = 0; k < 12; k++) {
         v[k] = in[k * cs + gid];
-        mx = max(mx, max(mag_hi(v[k].x), mag_hi(v[k].y)));
-        any |= (unsigned)__double2loint(v[k].x) | (unsigned)__double2loint(v[k].y);
+        const unsigned m = max(mag_hi(v[k].x), mag_hi(v[k].y));
+        mx = max(mx, m);
+        if (m | (unsigned)__double2loint(v[k].x) | (unsigned)__double2loint(v[k].y)) mn = min(mn, m);
     }
     const int em = (int)(mx >> 20);
     int e = em;
-    if (em > kMaxExp || (em < kMinExp && (mx | any))) e = kFxRaw;
-    else if (em < kMinExp) e = kFxZero;
+    if (mn == ~0u) e = kFxZero;
+    else if (em > kMaxExp || em < kMinExp || (int)(mn >> 20) < em - kKeep) e = kFxRaw;
 #pragma unroll
     for (int k = 0; k < 12; k++) {
         longlong2 o;

@@ -29,7 +29,7 @@ __device__ __forceinline__ void coords_full(const Geom &g, long long i, int &t, 
 
 __global__ void k_pack_links(const double2 *lex, Geom g, double2 *l64e, double2 *l64o,
                              float2 *l32fe, float2 *l32fo, float4 *l32ce, float4 *l32co,
-                             int *not_unitary)
+                             int *odd)
 {
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= g.V * 4) return;
@@ -49,16 +49,22 @@ __global__ void k_pack_links(const double2 *lex, Geom g, double2 *l64e, double2 
     double2 v[9];
 #pragma unroll
     for (int k = 0; k < 9; k++) v[k] = u[k];
+    // norms of the rows and columns, to a few digits, and the smallest entry by
+    // the larger of its parts
+    float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f}, least = 1.f;
 #pragma unroll
-    for (int a = 0; a < 3; a++) {  // row norms, to a few digits
-        float nn = 0.f;
+    for (int a = 0; a < 3; a++)
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            const float re = (float)v[3 * a + b].x, im = (float)v[3 * a + b].y;
-            nn = fmx(re, re, fmx(im, im, nn));
+            const float re = (float)v[3 * a + b].x, im = (float)v[3 * a + b].y, n2 = fmx(re, re, im * im);
+            row[a] += n2;
+            col[b] += n2;
+            least = fminf(least, fmaxf(fabsf(re), fabsf(im)));
         }
-        if (!(fabsf(nn - 1.f) <= 1e-3f)) atomicOr(not_unitary, 1);
-    }
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        if (!(fabsf(row[a] - 1.f) <= 1e-3f && fabsf(col[a] - 1.f) <= 1e-3f)) atomicOr(&odd[0], 1);
+    if (least < 0x1p-12f) atomicAdd(&odd[1], 1);
 #pragma unroll
     for (int k = 0; k < 9; k++) o64[k * g.Vh] = v[k];
 #pragma unroll
@@ -373,12 +379,12 @@ __global__ void k_cpp_commit(const double *src, double *dst, int T, int accumula
 }  // namespace
 
 cudaError_t launch_pack_links(const double2 *lex, const Geom &g, double2 *l64[2], float2 *l32f[2],
-                              float4 *l32c[2], int *not_unitary, cudaStream_t st)
+                              float4 *l32c[2], int *odd, cudaStream_t st)
 {
     const int block = 128;
     const long long n = g.V * 4;
     k_pack_links<<<(unsigned)((n + block - 1) / block), block, 0, st>>>(
-        lex, g, l64[0], l64[1], l32f[0], l32f[1], l32c[0], l32c[1], not_unitary);
+        lex, g, l64[0], l64[1], l32f[0], l32f[1], l32c[0], l32c[1], odd);
     return cudaGetLastError();
 }
 

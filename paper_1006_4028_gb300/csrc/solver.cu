@@ -309,7 +309,7 @@ dp_status Batch::init()
     op64.links[1] = f->l64[1];
     op64.hop = hop64_d;
     op64.nrhs = n;
-    if (f->unitary) {
+    if (f->fx) {
         // the integer kernel's exponents; its converted input goes to to64,
         // which holds a job's source only while the job is set up or finished.
         // Without the memory (8 bytes per site and RHS to the vectors' 2000)
@@ -1593,7 +1593,7 @@ dp_status dp_schur_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile *
     void *hd = c.alloc(tb), *had = c.alloc(tb), *tp = c.alloc(vb), *tq = c.alloc(vb);
     // FP64: exponents for the integer kernel (without them the FP64 kernel serves)
     const size_t ne = (size_t)g.Vh * nrhs;
-    int *ex = pr == 0 && f.unitary ? (int *)c.alloc(2 * ne * sizeof(int)) : nullptr;
+    int *ex = pr == 0 && f.fx ? (int *)c.alloc(2 * ne * sizeof(int)) : nullptr;
     if (ex) {
         op.xw = tp;
         op.xe = ex;

@@ -312,10 +312,10 @@ dp_status Batch::init()
     if (f->fx) {
         // the integer kernel's exponents; its converted input goes to to64,
         // which holds a job's source only while the job is set up or finished.
-        // Without the memory (8 bytes per site and RHS to the vectors' 2000)
-        // the FP64 kernel serves.
+        // Without the memory (8 to 12 bytes per site and RHS to the vectors'
+        // 2000) the FP64 kernel serves.
         const size_t ne = (size_t)Vh * n;
-        int *ex = (int *)get(2 * ne * sizeof(int));
+        int *ex = (int *)get((ipr == 0 ? 3 : 2) * ne * sizeof(int));
         if (ex) {
             op64.xw = to64;
             op64.xe = ex;
@@ -327,6 +327,10 @@ dp_status Batch::init()
     opin.pr = ipr;
     opin.lf = ilf;
     if (ipr != 0) opin.xw = nullptr;
+    // t64 and its exponents outlive the round (harvest rebuilds the other
+    // parity from them, also for an RHS that the next inner solve switched off
+    // as not finite), so the inner solver's intermediate vector has its own
+    if (opin.xw) opin.te = op64.te + (size_t)Vh * n;
     for (int p = 0; p < 2; p++) {
         dp_status e = field_links(c, *f, ilf, p, &opin.links[p]);
         if (e != DP_OK) return e;

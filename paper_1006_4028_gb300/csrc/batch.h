@@ -76,6 +76,10 @@ class Batch {
     Batch &operator=(const Batch &) = delete;
 
     static size_t bytes_needed(const Geom &g, int nslots, int prec);
+    // on top of that where the FP64 operator runs in integer arithmetic
+    // (Field::fx); a batch told not to (before init) takes the FP64 kernel
+    static size_t fx_bytes(const Geom &g, int nslots, int prec);
+    void set_fx(bool on) { use_fx = on; }
     dp_status init();
     bool can_admit(int ncomp) const;
     // set up the job's source, Schur right-hand side and outer state
@@ -134,6 +138,7 @@ class Batch {
     int round_iters;
     int sp = 0;
     int max_jobs = 0;
+    bool use_fx = true;
     std::function<bool()> yield_check;
     int yield_min = 8;
     int mixed = 1, ipr = 1, ilf = LINK_F32_12;

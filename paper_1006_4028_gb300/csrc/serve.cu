@@ -46,6 +46,7 @@ struct Worker {
     std::unique_ptr<Batch> B;
     std::thread th;
     size_t bytes = 0;
+    bool fx = false;       // the batch's budget holds the integer operator's scratch
     bool stop = false;     // set by the coordinator (under Scheduler::mu)
     bool finished = false; // the thread has left its loop
     int running = 0;       // jobs in the batch (under Scheduler::mu)
@@ -173,6 +174,7 @@ void Scheduler::work(Worker *w)
             w->running = 0;
             lk.unlock();
             w->B.reset(new Batch(c, w->field, max_slots, opts, 200, 0, true));
+            w->B->set_fx(w->fx);
             dp_status e = w->B->init();
             install_yield(w);
             lk.lock();
@@ -198,15 +200,19 @@ void Scheduler::run()
             if (workers.count(fid)) continue;
             const size_t need = Batch::bytes_needed(rq->field->g, max_slots, rq->req.prec);
             if (in_use + need > budget) continue;
+            const Field &fd = *rq->field;
+            const size_t fx = fd.fx ? Batch::fx_bytes(fd.g, max_slots, rq->req.prec) : 0;
             auto w = std::make_unique<Worker>();
             w->fid = fid;
             w->field = rq->field;
-            w->bytes = need;
-            in_use += need;
+            w->fx = in_use + need + fx <= budget;
+            w->bytes = w->fx ? need + fx : need;
+            in_use += w->bytes;
             Worker *wp = w.get();
             workers.emplace(fid, std::move(w));
             lk.unlock();
             wp->B = std::make_unique<Batch>(c, wp->field, max_slots, opts, 200, 0, true);
+            wp->B->set_fx(wp->fx);
             dp_status s = wp->B->init();
             std::string msg = s != DP_OK ? dp_last_error() : "";
             lk.lock();

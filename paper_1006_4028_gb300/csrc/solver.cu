@@ -215,6 +215,11 @@ size_t Batch::bytes_needed(const Geom &g, int nslots, int prec)
     return 6 * v64 + 8 * vin + shadow + ((size_t)1 << 20);
 }
 
+size_t Batch::fx_bytes(const Geom &g, int nslots, int prec)
+{
+    return (size_t)g.Vh * nslots * sizeof(int) * (prec == DP_PREC_FP64 ? 3 : 2);
+}
+
 dp_status Batch::init()
 {
     const Geom &g = f->g;
@@ -309,28 +314,10 @@ dp_status Batch::init()
     op64.links[1] = f->l64[1];
     op64.hop = hop64_d;
     op64.nrhs = n;
-    if (f->fx) {
-        // the integer kernel's exponents; its converted input goes to to64,
-        // which holds a job's source only while the job is set up or finished.
-        // Without the memory (8 to 12 bytes per site and RHS to the vectors'
-        // 2000) the FP64 kernel serves.
-        const size_t ne = (size_t)Vh * n;
-        int *ex = (int *)get((ipr == 0 ? 3 : 2) * ne * sizeof(int));
-        if (ex) {
-            op64.xw = to64;
-            op64.xe = ex;
-            op64.te = ex + ne;
-        }
-    }
     set_shape(op64, c->launch_shape(Vh, 0, LINK_F64_18, n));
     opin = op64;
     opin.pr = ipr;
     opin.lf = ilf;
-    if (ipr != 0) opin.xw = nullptr;
-    // t64 and its exponents outlive the round (harvest rebuilds the other
-    // parity from them, also for an RHS that the next inner solve switched off
-    // as not finite), so the inner solver's intermediate vector has its own
-    if (opin.xw) opin.te = op64.te + (size_t)Vh * n;
     for (int p = 0; p < 2; p++) {
         dp_status e = field_links(c, *f, ilf, p, &opin.links[p]);
         if (e != DP_OK) return e;
@@ -377,6 +364,25 @@ dp_status Batch::init()
             if (e != DP_OK) return e;
         }
         opdf.hop = hopdf_d;
+    }
+    if (use_fx && f->fx) {
+        // the integer kernel's exponents; its converted input goes to to64,
+        // which holds a job's source only while the job is set up or finished.
+        // Allocated last, so that no vector goes without; without them the FP64
+        // kernel serves.  t64 and its exponents outlive the round (harvest
+        // rebuilds the other parity from them, also for an RHS that the next
+        // inner solve switched off as not finite), so the inner solver's
+        // intermediate vector has its own.
+        const size_t ne = (size_t)Vh * n;
+        int *ex = (int *)get(fx_bytes(g, n, opts.prec));
+        if (ex) {
+            for (Op *o : {&op64, &opin, &opin_adj}) {
+                if (o->pr != 0) continue;
+                o->xw = to64;
+                o->xe = ex;
+                o->te = o == &op64 ? ex + ne : ex + 2 * ne;
+            }
+        }
     }
     check_every = opts.check_every > 0 ? opts.check_every : (Vh * n >= (1 << 20) ? 2 : 8);
     if (own_stream_) {

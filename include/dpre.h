@@ -404,6 +404,9 @@ dp_status dp_fit_correlator(const double *c, int T, int kind, int t0, int t1, do
  * per SM (64, 96 or 128 threads per block); all of 2-6 need 2 RHS per
  * thread and FP32 or 16-bit 12-real links (6 also takes FP32 18-real
  * links).  -1: the tuned or default choice.
+ * FP64 in integer arithmetic (see dp_prec) divides its work by itself: the
+ * shape is checked but serves the fields it does not take; the time includes
+ * the conversion of `in`, once a launch.
  * FP32 needs nrhs even.  iters launches back to back; if ms_out is non-NULL
  * it receives the average launch time measured with CUDA events on the
  * context stream. */
@@ -433,7 +436,7 @@ dp_status dp_schur_dev(dp_ctx *ctx, dp_field field, double M, const dp_profile *
 /* Time candidate launch shapes of the multi-RHS dslash for this field,
  * precision and nrhs (64-256 threads per block x the RHS-per-thread and
  * staging choices of dp_dslash_dev), and keep the fastest for the solver's
- * later launches.  best_* may be NULL.  DP_ERR_INVALID_ARG if no shape serves
+ * later launches (FP64 in integer arithmetic: the one launch there is).  best_* may be NULL.  DP_ERR_INVALID_ARG if no shape serves
  * nrhs (FP32 with an odd count). */
 dp_status dp_autotune(dp_ctx *ctx, dp_field field, int prec, int compress12, int nrhs,
                       int *best_block_threads, int *best_rhs_per_thread, int *best_stages,

@@ -971,13 +971,24 @@ dp_status dp_autotune(dp_ctx *ctx, dp_field field, int prec, int compress12, int
         set_error("out of device memory (autotune)");
         return DP_ERR_OOM;
     }
-    cudaMemsetAsync(in, 0, vb, c.stream);
+    // (the FP64 operator passes over neighbours that are zero)
+    const cudaError_t fill = pr == 0 ? launch_tuner_input((double *)in, (long long)(vb / sizeof(double)), c.stream)
+                                     : cudaMemsetAsync(in, 0, vb, c.stream);
+    if (fill != cudaSuccess) {
+        c.release(in);
+        c.release(out);
+        set_error("filling the tuner's input: %s", cudaGetErrorString(fill));
+        return DP_ERR_CUDA;
+    }
     // candidates: four block sizes x RHS per thread (FP64: 1; FP32: one or
     // two RHS pairs) x how neighbour data arrives (FP32 one pair per thread:
     // direct, shared-memory staging of spinor and link 2-3 directions ahead
     // or in a persistent wave, direct with an L1 prefetch 2 directions ahead,
     // or the spinor alone staged 2 directions ahead with the link from L1)
-    const int blocks[] = {64, 96, 128, 192, 256};
+    // (the integer FP64 kernel divides its work by itself: one candidate, whose
+    // shape serves the scalar kernel)
+    std::vector<int> blocks = {64, 96, 128, 192, 256};
+    if (pr == 0 && fp->fx) blocks = {64};
     const int rpts[] = {1, 2, 4};
     const int stage_opts[] = {0, 2, 3, 4, 5, 6};
     Shape best;

@@ -128,6 +128,9 @@ cudaError_t launch_to_df(const double2 *in, float4 *out, long long count, const 
 cudaError_t launch_from_df(const float4 *in, double2 *out, long long count, const int *mask, int n,
                            int mask_stride, cudaStream_t st);
 
+// n doubles spread over [-1, 1), the tuner's FP64 spinor
+cudaError_t launch_tuner_input(double *v, long long n, cudaStream_t st);
+
 // launch shape of the Schur dslash launches (tuner result or default)
 struct Shape {
     int block = 64;

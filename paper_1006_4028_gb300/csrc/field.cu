@@ -492,6 +492,24 @@ cudaError_t launch_restore_contract(const double2 *xe, const double2 *xo, const 
     return cudaGetLastError();
 }
 
+namespace {
+__global__ void k_tuner_input(double *v, long long n)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    unsigned long long z = 0x9e3779b97f4a7c15ull * (unsigned long long)(i + 1);  // splitmix64
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    v[i] = (double)(long long)(z ^ (z >> 31)) * 0x1p-63;
+}
+}  // namespace
+
+cudaError_t launch_tuner_input(double *v, long long n, cudaStream_t st)
+{
+    k_tuner_input<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(v, n);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_cpp_commit(const double *src, double *dst, int T, int accumulate, cudaStream_t st)
 {
     k_cpp_commit<<<(T + 127) / 128, 128, 0, st>>>(src, dst, T, accumulate);

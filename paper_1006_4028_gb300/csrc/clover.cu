@@ -227,7 +227,6 @@ __device__ __forceinline__ bool invert_block(const double *m, double diag, doubl
         const C d = X[col * 6 + col];
         const double den = d.re * d.re + d.im * d.im;
         const C pinv = {d.re / den, -d.im / den};
-        X[col * 6 + col] = {1.0, 0.0};
 #pragma unroll
         for (int j = 0; j < 6; j++) X[col * 6 + j] = j == col ? pinv : cmul(pinv, X[col * 6 + j]);
 #pragma unroll

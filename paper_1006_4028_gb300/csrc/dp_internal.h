@@ -23,6 +23,7 @@ namespace dp {
 
 constexpr int kMaxRhs = 64;
 constexpr int kMaxL = 256;
+constexpr int kSms = 152;  // SMs of a GB300, for grids that should fill it
 
 struct Geom {
     int T, Lx, Ly, Lz, Lxh, Lmax;

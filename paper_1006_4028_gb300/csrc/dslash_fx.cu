@@ -731,7 +731,7 @@ cudaError_t launch_dslash_fx(const DslashParams &p, int epi, cudaStream_t st)
             best = k;
         }
     }
-    constexpr long long kFill = 2 * 152;
+    constexpr long long kFill = 2 * kSms;
     const long long fine = (p.g.Vh + kFill - 1) / kFill;
     fl.sites = (int)(fine < best ? fine : best);
     // the distinct groups of the launch

@@ -449,7 +449,7 @@ cudaError_t launch_contract_hl(const double2 *xe, const double2 *xo, const Geom 
 int contract_blocks_per_slice(const Geom &g)
 {
     const long long Vs = g.Vh / g.T;
-    const long long fill = (4 * 152 + g.T - 1) / g.T, most = (Vs + 31) / 32;
+    const long long fill = (4 * kSms + g.T - 1) / g.T, most = (Vs + 31) / 32;
     long long P = std::max((Vs + 1023) / 1024, std::min(fill, most));
     if (P < 1) P = 1;
     if (P > 64) P = 64;

@@ -13,9 +13,12 @@
 // partials and the FP64 conversions around them took most of a reduction
 // kernel on a small lattice (16x8^3, 12 RHS: the three of a BiCGStab iteration
 // 20, 17 and 16 us, with integers 16, 13 and 10).  An integer add with
-// alignment is about 10 instructions.  Terms are aligned to the largest
-// one with its leading bit at 2^kLead or above, so a sum of N terms is off by
-// at most N 2^-kLead of its largest term (FP64 adds: N 2^-53 of the sum).
+// alignment is about 10 instructions.  A block's terms have their leading bit at
+// lead_for(lanes) (53 at 256 lanes, 60 at 2) and are aligned to the largest one,
+// each addition rounding down by a unit at most: off by lanes 2^-lead_for(lanes)
+// of the largest term.  The block's total keeps lead_for(grid) bits (50 at 1216
+// blocks, 53 at 152), and the last block's sum is off by 2 grid 2^-lead_for(grid)
+// of the largest total, half of that expected.  (FP64 adds: N 2^-53 of the sum.)
 #pragma once
 
 #include <cuda_runtime.h>

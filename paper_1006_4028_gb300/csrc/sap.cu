@@ -300,7 +300,7 @@ template <int LF>
 cudaError_t launch_sap_k(const SapParams &p, dim3 grid, int threads, size_t smem, cudaStream_t st)
 {
     static const cudaError_t attr =
-        cudaFuncSetAttribute(k_sap_block<LF>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+        cudaFuncSetAttribute(k_sap_block<LF>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024);
     if (attr != cudaSuccess) return attr;
     k_sap_block<LF><<<grid, threads, smem, st>>>(p);
     return cudaGetLastError();

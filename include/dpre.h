@@ -460,7 +460,8 @@ dp_status dp_timing_enable(dp_ctx *ctx, int on);
 dp_status dp_timing_reset(dp_ctx *ctx);
 /* Statistics of kernel class `name`: launches and total milliseconds of
  * stream time while timing is on.  Classes: "dslash_fp32", "dslash_fp64",
- * "dslash_df" (operator launches), "clover_apply", "sap_block", the inner
+ * "dslash_df" (operator launches, FP64 with the conversion of the input),
+ * "clover_apply", "sap_block", the inner
  * solvers' BLAS passes ("blas_alpha", "blas_s", "blas_omega", "blas_update",
  * "blas_p"), "outer_blas", "slice_norms", and the solver phases "admit",
  * "round", "harvest".  Synchronises the stream. */

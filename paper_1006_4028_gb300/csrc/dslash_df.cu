@@ -7,8 +7,8 @@
 // two-sum, the low parts plainly added) and are normalised once per use.
 // GB300 runs FP32 at 64 times its FP64 rate, so this replaces the FP64
 // dslash of the true-residual recomputation where 1e-14 relative accuracy
-// suffices (residues r >= 1e-12).  At 48x24^3, 12 RHS it takes 4.25 ms a launch
-// against 7.4 for the scalar FP64 kernel and 2.3 for the integer one
+// suffices (residues r >= 1e-12).  At 48x24^3, 12 RHS it takes 4.36 ms a launch
+// against 7.4 for the scalar FP64 kernel and 2.5 for the integer one
 // (dslash_fx.cu), whose results are FP64: a choice for links the integers do
 // not take.
 //

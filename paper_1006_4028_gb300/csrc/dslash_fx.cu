@@ -62,12 +62,13 @@
 // spinor eight times) cost 13 integer instructions or one 68-cycle cvt per
 // real and 48 registers for the raw spinor: 0.61 ms for 12 RHS on 32x16^3.
 // Converting once (k_to_fx, a pass at copy rate: 0.04 ms) leaves the hop kernel
-// with adds and products: 0.42 ms (x - A^-1 D: 0.46, its 24 FP64 subtractions on the FP64
-// pipe) where k_dslash64 takes 1.36.  48x24^3: 2.3 ms with the conversion
-// against 7.4; one RHS on 32x16^3 0.12 against 0.24.  What holds it now is latency: 10.4
-// thousand instructions a warp, four warps a quarter (128 registers: 24 int64
+// with adds and products.  A^-1 D with the conversion, all RHS active: 12 RHS on
+// 32x16^3 0.55 ms where k_dslash64 takes 1.49, on 48x24^3 2.72 against 7.40
+// (x - A^-1 D 0.1 more: its 24 subtractions are on the FP64 pipe), one RHS on
+// 32x16^3 0.117 against 0.150.  What holds it now is latency: 10.5 thousand
+// instructions a warp, four warps a quarter (128 registers: 24 int64
 // accumulators alone are 48), 0.41 of the issue slots, fixed-latency waits
-// first; at 96 registers for five warps it spills and takes 0.63.
+// first; at 96 registers for five warps it spills and took a half more.
 //
 // Layout of the work: a block holds whole sites, all right-hand sides of each,
 // one thread per (site, RHS).  The limbs of a direction's links (and of a
